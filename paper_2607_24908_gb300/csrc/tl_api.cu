@@ -207,6 +207,8 @@ int finish_create(tl_lattice *L, int N, double kIR, int nf, tl_dtype dtype, cons
     int dev = 0;
     TL_CK(cudaGetDevice(&dev));
     TL_CK(cudaDeviceGetAttribute(&L->sm_count, cudaDevAttrMultiProcessorCount, dev));
+    L->device = dev;
+    tl::scratch_user(dev, 1);
     L->tuning = tl::default_tuning(N, nf, (int)L->esz);
     L->geom = tl::pass_geometry(N, (int)L->esz, L->sm_count, nf, L->tuning);
     TL_CK(cudaMalloc(&L->d_sc, sizeof(Scalars)));
@@ -306,6 +308,10 @@ int shared_plan(int N, cufftType type, cudaStream_t s, SharedPlan **out)
     if (it == g_plans.end()) {
         SharedPlan p{};
         cufftResult r = cufftPlan3d(&p.h, N, N, N, type);
+        if (r != CUFFT_SUCCESS) {  // perhaps for memory that the scratch pool keeps
+            tl::scratch_release(dev);
+            r = cufftPlan3d(&p.h, N, N, N, type);
+        }
         if (r != CUFFT_SUCCESS) return fail(TL_ECUDA, "cufftPlan3d(%d) failed (%d)", N, (int)r);
         cudaError_t e = cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming);
         if (e != cudaSuccess) {
@@ -386,8 +392,8 @@ int tl_lattice_create(tl_lattice **out, int N, double kIR, int n_fields, tl_dtyp
     // pass do not sit at identical offsets modulo large powers of two.
     const size_t stagger = array_stagger();
     const size_t bytes = tl_state_bytes(N, n_fields, dtype) + 4 * (size_t)n_fields * stagger;
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    size_t free_b = 0;
+    if (tl::free_device_bytes(bytes + (64u << 20), &free_b) != cudaSuccess) {
         delete L;
         return fail(TL_ECUDA, "cudaMemGetInfo failed (no CUDA device?)");
     }
@@ -462,6 +468,7 @@ void tl_lattice_destroy(tl_lattice *L)
     if (L->own && L->base) cudaFree(L->base);
     if (L->d_sc) cudaFree(L->d_sc);
     if (L->d_slots) cudaFree(L->d_slots);
+    if (L->device >= 0) tl::scratch_user(L->device, -1);
     delete L;
 }
 
@@ -790,8 +797,8 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
     const cufftHandle plan = sp->h;
     double2 *modes = nullptr;
     double *real = nullptr;
-    TL_CK(cudaMallocAsync((void **)&modes, nh * sizeof(double2), L->stream));
-    cudaError_t e = cudaMallocAsync((void **)&real, n3 * sizeof(double), L->stream);
+    TL_CK(tl::scratch_alloc((void **)&modes, nh * sizeof(double2), L->stream));
+    cudaError_t e = tl::scratch_alloc((void **)&real, n3 * sizeof(double), L->stream);
     if (e != cudaSuccess) {
         cudaFreeAsync(modes, L->stream);
         return fail(TL_ENOMEM, "scratch allocation for the initial field failed");
@@ -860,9 +867,9 @@ int tl_spectrum(tl_lattice *L, int field, int which, int nbins, double *k, doubl
     const cufftHandle plan = sp->h;
     double2 *modes = nullptr;
     double *real = nullptr, *acc = nullptr;
-    TL_CK(cudaMallocAsync((void **)&modes, nh * sizeof(double2), L->stream));
-    TL_CK(cudaMallocAsync((void **)&real, n3 * sizeof(double), L->stream));
-    TL_CK(cudaMallocAsync((void **)&acc, (size_t)nb * 3 * sizeof(double), L->stream));
+    TL_CK(tl::scratch_alloc((void **)&modes, nh * sizeof(double2), L->stream));
+    TL_CK(tl::scratch_alloc((void **)&real, n3 * sizeof(double), L->stream));
+    TL_CK(tl::scratch_alloc((void **)&acc, (size_t)nb * 3 * sizeof(double), L->stream));
     TL_CK(cudaMemsetAsync(acc, 0, (size_t)nb * 3 * sizeof(double), L->stream));
     TL_CK(tl::launch_widen((int)L->dtype, real, L->buf[L->cur][which][field], n3, N, L->model.pitch, L->model.pplane,
                            L->sm_count, L->stream));

@@ -206,6 +206,17 @@ cudaError_t launch_pass(int dtype, const Model &m, const FieldPtrs &fp, const Pa
                         Scalars *sc, double *slots, bool measure_only, cudaStream_t s,
                         const TmaMaps *maps = nullptr);
 
+// Scratch memory on the current device, ordered on s (freed with
+// cudaFreeAsync), from the library's pool (tl_scratch.cu).
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s);
+// Give back what device dev's pool keeps unused.
+void scratch_release(int dev);
+// A lattice of device dev comes (+1) or goes (-1); with the last one the pool
+// gives its memory back.
+void scratch_user(int dev, int change);
+// Free bytes of the current device, after scratch_release if fewer than need are.
+cudaError_t free_device_bytes(size_t need, size_t *free_b);
+
 // Record msg+detail as this thread's tl_last_error() text; returns code.
 int set_error(int code, const char *msg, const char *detail);
 

@@ -32,6 +32,7 @@ struct tl_lattice {
     tl::PassGeom geom{};
     tl::Model model{};
     int sm_count = 0;
+    int device = -1;              // counted there as a user of the scratch pool
     int64_t step = 0;
     int64_t langevin_steps = 0;  // Langevin steps since the last state reset (noise counters)
     bool energies_valid = false;

@@ -785,12 +785,12 @@ int tl_su2_create(tl_su2 **out, int N, tl_dtype dtype, void *cuda_stream)
     Y->esz = dtype == TL_F32 ? 4 : 8;
     Y->stream = static_cast<cudaStream_t>(cuda_stream);
     const size_t n3 = (size_t)N * N * N;
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    const size_t need = 33 * n3 * Y->esz;  // two link buffers (12 values a site each) and the fields (9)
+    size_t free_b = 0;
+    if (tl::free_device_bytes(need + (64u << 20), &free_b) != cudaSuccess) {
         delete Y;
         return tl::fail(TL_ECUDA, "cudaMemGetInfo failed (no CUDA device?)");
     }
-    const size_t need = 33 * n3 * Y->esz;  // two link buffers (12 values a site each) and the fields (9)
     if (need + (64u << 20) > free_b) {
         delete Y;
         return tl::fail(TL_ENOMEM, "SU(2) lattice needs %zu bytes", need);

@@ -162,8 +162,8 @@ int tl_set_potential(tl_lattice *lat, const tl_potential *pot);
  * Sec. 3.5); the spectrum A/(2 omega_k) is the workloads' vacuum spectrum.
  * Draw the initial state (see tl_init_spec), set a = a0 and, when expanding,
  * b = a0^(1+alpha) sqrt(mu2 rho0/3) with rho0 the lattice-averaged K+G+V of
- * that state.  Uses cuFFT (c2r, FP64) and temporary device memory of about
- * 16 N^3 bytes, from a pool of the library's that keeps up to 1 GiB of it (and
+ * that state.  Uses cuFFT (complex, FP64) and temporary device memory of about
+ * 8 N^3 bytes, from a pool of the library's that keeps up to 1 GiB of it (and
  * of tl_spectrum's) per device between calls, until the device's last lattice
  * is destroyed.  Resets step and time to 0. */
 int tl_init_fluctuations(tl_lattice *lat, uint64_t seed, const tl_init_spec *spec);

@@ -9,9 +9,9 @@
 #include <string.h>
 
 #include <map>
-#include <tuple>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "tl_fourier.cuh"
@@ -286,8 +286,8 @@ int check_field(const tl_lattice *L, int field, int which)
     return TL_OK;
 }
 
-// cuFFT plans shared by all lattices of a size on a device (planning costs
-// milliseconds and a workspace per plan).  Under this mutex a plan is bound
+// cuFFT plans (N x N x N/2 complex, see tl_fourier.cuh) shared by all lattices
+// of a size on a device (planning costs milliseconds and a workspace per plan).  Under this mutex a plan is bound
 // to the caller's stream, which first waits for the plan's previous
 // executions (on whatever stream they were enqueued) through the plan's
 // event; the caller records that event after its last execution.  Calls that
@@ -297,20 +297,20 @@ struct SharedPlan {
     cudaEvent_t done;  // recorded after the latest enqueued execution
 };
 std::mutex g_plan_mu;
-std::map<std::tuple<int, int, int>, SharedPlan> g_plans;  // (device, N, cufftType) -> plan
+std::map<std::pair<int, int>, SharedPlan> g_plans;  // (device, N) -> plan
 
-int shared_plan(int N, cufftType type, cudaStream_t s, SharedPlan **out)
+int shared_plan(int N, cudaStream_t s, SharedPlan **out)
 {
     int dev = 0;
     TL_CK(cudaGetDevice(&dev));
-    auto key = std::make_tuple(dev, N, (int)type);
+    auto key = std::make_pair(dev, N);
     auto it = g_plans.find(key);
     if (it == g_plans.end()) {
         SharedPlan p{};
-        cufftResult r = cufftPlan3d(&p.h, N, N, N, type);
+        cufftResult r = cufftPlan3d(&p.h, N, N, N / 2, CUFFT_Z2Z);
         if (r != CUFFT_SUCCESS) {  // perhaps for memory that the scratch pool keeps
             tl::scratch_release(dev);
-            r = cufftPlan3d(&p.h, N, N, N, type);
+            r = cufftPlan3d(&p.h, N, N, N / 2, CUFFT_Z2Z);
         }
         if (r != CUFFT_SUCCESS) return fail(TL_ECUDA, "cufftPlan3d(%d) failed (%d)", N, (int)r);
         cudaError_t e = cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming);
@@ -786,23 +786,16 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
     if (!L->has_pot) return fail(TL_ESTATE, "tl_set_potential must come first (b0 needs the potential)");
     if (!(spec->A >= 0.0) || !isfinite(spec->A)) return fail(TL_EINVAL, "A must be finite and >= 0");
     const int N = L->N;
-    const size_t n3 = n3_of(N);
-    const size_t nh = (size_t)N * N * (N / 2 + 1);
     std::lock_guard<std::mutex> plan_lock(g_plan_mu);
     SharedPlan *sp = nullptr;
     {
-        int prc = shared_plan(N, CUFFT_Z2D, L->stream, &sp);
+        int prc = shared_plan(N, L->stream, &sp);
         if (prc) return prc;
     }
     const cufftHandle plan = sp->h;
-    double2 *modes = nullptr;
-    double *real = nullptr;
-    TL_CK(tl::scratch_alloc((void **)&modes, nh * sizeof(double2), L->stream));
-    cudaError_t e = tl::scratch_alloc((void **)&real, n3 * sizeof(double), L->stream);
-    if (e != cudaSuccess) {
-        cudaFreeAsync(modes, L->stream);
+    double2 *modes = nullptr;  // N x N x N/2 modes, then (in place) the N^3 field
+    if (tl::scratch_alloc((void **)&modes, n3_of(N) * sizeof(double), L->stream) != cudaSuccess)
         return fail(TL_ENOMEM, "scratch allocation for the initial field failed");
-    }
     int rc = TL_OK;
     const bool expanding = L->ex.expanding != 0;
     const double pscale = expanding ? pow(L->ex.a0, 3.0 - L->ex.alpha) : 1.0;
@@ -816,14 +809,15 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
                                                        spec->fixed_modulus ? 1 : 0, seed, which == 0 ? (uint64_t)f : (uint64_t)(8 + f),
                                                        L->sm_count, L->stream);
                 if (ce != cudaSuccess) { rc = fail(TL_ECUDA, "fill_modes: %s", cudaGetErrorString(ce)); break; }
-                cufftResult fr = cufftExecZ2D(plan, reinterpret_cast<cufftDoubleComplex *>(modes), real);
-                if (fr != CUFFT_SUCCESS) { rc = fail(TL_ECUDA, "cufftExecZ2D failed (%d)", (int)fr); break; }
-                ce = tl::launch_assemble((int)L->dtype, dst, real, n3, base, which == 0 ? 1.0 : pscale, N,
-                                         L->model.pitch, L->model.pplane, L->sm_count, L->stream);
+                cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
+                cufftResult fr = cufftExecZ2Z(plan, z, z, CUFFT_INVERSE);
+                if (fr != CUFFT_SUCCESS) { rc = fail(TL_ECUDA, "cufftExecZ2Z failed (%d)", (int)fr); break; }
+                ce = tl::launch_assemble((int)L->dtype, dst, reinterpret_cast<double *>(modes), base,
+                                         which == 0 ? 1.0 : pscale, N, L->model.pitch, L->model.pplane, L->stream);
                 if (ce != cudaSuccess) { rc = fail(TL_ECUDA, "assemble: %s", cudaGetErrorString(ce)); break; }
             } else {
-                cudaError_t ce = tl::launch_assemble((int)L->dtype, dst, nullptr, n3, base, 0.0, N, L->model.pitch,
-                                                     L->model.pplane, L->sm_count, L->stream);
+                cudaError_t ce = tl::launch_assemble((int)L->dtype, dst, nullptr, base, 0.0, N, L->model.pitch,
+                                                     L->model.pplane, L->stream);
                 if (ce != cudaSuccess) { rc = fail(TL_ECUDA, "assemble: %s", cudaGetErrorString(ce)); break; }
             }
         }
@@ -833,12 +827,7 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
         if (re != cudaSuccess && rc == TL_OK) rc = fail(TL_ECUDA, "cudaEventRecord: %s", cudaGetErrorString(re));
     }
     cudaFreeAsync(modes, L->stream);
-    cudaFreeAsync(real, L->stream);
     if (rc) return rc;
-    for (int f = 0; f < L->nf; ++f)
-        for (int which = 0; which < 2; ++which)
-            TL_CK(tl::launch_fill_ghosts((int)L->dtype, L->buf[L->cur][which][f], N, L->model.pitch, L->model.pplane,
-                                         L->stream));
     L->state_mask = (1u << (2 * L->nf)) - 1u;
     L->has_state = true;
     L->step = 0;
@@ -856,32 +845,29 @@ int tl_spectrum(tl_lattice *L, int field, int which, int nbins, double *k, doubl
     const int N = L->N;
     const int nb = tl_spectrum_bins(N);
     if (nbins < nb) return fail(TL_EINVAL, "nbins must be >= %d", nb);
-    const size_t n3 = n3_of(N);
-    const size_t nh = (size_t)N * N * (N / 2 + 1);
     std::lock_guard<std::mutex> plan_lock(g_plan_mu);
     SharedPlan *sp = nullptr;
     {
-        int prc = shared_plan(N, CUFFT_D2Z, L->stream, &sp);
+        int prc = shared_plan(N, L->stream, &sp);
         if (prc) return prc;
     }
     const cufftHandle plan = sp->h;
-    double2 *modes = nullptr;
-    double *real = nullptr, *acc = nullptr;
-    TL_CK(tl::scratch_alloc((void **)&modes, nh * sizeof(double2), L->stream));
-    TL_CK(tl::scratch_alloc((void **)&real, n3 * sizeof(double), L->stream));
+    double2 *modes = nullptr;  // the field, then (in place) its N x N x N/2 modes
+    double *acc = nullptr;
+    TL_CK(tl::scratch_alloc((void **)&modes, n3_of(N) * sizeof(double), L->stream));
     TL_CK(tl::scratch_alloc((void **)&acc, (size_t)nb * 3 * sizeof(double), L->stream));
     TL_CK(cudaMemsetAsync(acc, 0, (size_t)nb * 3 * sizeof(double), L->stream));
-    TL_CK(tl::launch_widen((int)L->dtype, real, L->buf[L->cur][which][field], n3, N, L->model.pitch, L->model.pplane,
-                           L->sm_count, L->stream));
-    cufftResult fr = cufftExecD2Z(plan, real, reinterpret_cast<cufftDoubleComplex *>(modes));
-    if (fr != CUFFT_SUCCESS) return fail(TL_ECUDA, "cufftExecD2Z failed (%d)", (int)fr);
+    TL_CK(tl::launch_widen((int)L->dtype, reinterpret_cast<double *>(modes), L->buf[L->cur][which][field], N,
+                           L->model.pitch, L->model.pplane, L->stream));
+    cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
+    cufftResult fr = cufftExecZ2Z(plan, z, z, CUFFT_FORWARD);
+    if (fr != CUFFT_SUCCESS) return fail(TL_ECUDA, "cufftExecZ2Z failed (%d)", (int)fr);
     TL_CK(cudaEventRecord(sp->done, L->stream));
     TL_CK(tl::launch_bin(modes, N, nb, acc, acc + nb, reinterpret_cast<unsigned long long *>(acc + 2 * nb),
                          L->sm_count, L->stream));
     std::vector<double> h((size_t)nb * 3);
     TL_CK(cudaMemcpyAsync(h.data(), acc, h.size() * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
     cudaFreeAsync(modes, L->stream);
-    cudaFreeAsync(real, L->stream);
     cudaFreeAsync(acc, L->stream);
     TL_CK(cudaStreamSynchronize(L->stream));
     const double Lbox = 2.0 * M_PI / L->kIR;

@@ -2,7 +2,8 @@
 // loop).  The paper prepares states and measures in Fourier space through its
 // automatic Fourier views (Sec. 2) with Philox-2x64 random numbers (Sec. 2);
 // here the mode draw, the field assembly and the shell binning are kernels
-// of this library and the transforms are cuFFT library calls (FP64).
+// of this library and the transforms are cuFFT library calls (FP64, complex, of
+// half the real size: tl_fourier.cuh).
 #include <math.h>
 
 #include "tl_fourier.cuh"
@@ -10,105 +11,260 @@
 
 namespace tl {
 
-
 __device__ __forceinline__ int signed_mode(int i, int N) { return (i < N / 2) ? i : i - N; }
 
-// One entry of the half spectrum [iz][iy][ix], ix in [0, N/2].
-__global__ void fill_modes_kernel(double2 *modes, int N, double kIR, double A, double m2, int pi_spectrum,
-                                  int fixed_modulus, uint64_t seed, uint64_t stream)
+// exp(sign 2 pi i j/N), j = 0 .. N/4, into a CTA's shared table.
+__device__ __forceinline__ void fill_roots(double2 *root, int N, double sign)
 {
-    const int NH = N / 2 + 1;
-    const size_t total = (size_t)N * N * NH;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int ix = (int)(i % NH);
-        const int iy = (int)((i / NH) % N);
-        const int iz = (int)(i / ((size_t)NH * N));
-        const long nx = ix, ny = signed_mode(iy, N), nz = signed_mode(iz, N);
-        const long r2 = nx * nx + ny * ny + nz * nz;
-        double2 out = make_double2(0.0, 0.0);
-        if (r2 > 0 && 4 * r2 < (long)N * N) {
-            const bool canon = nx > 0 || (nx == 0 && (ny > 0 || (ny == 0 && nz > 0)));
-            const uint64_t own = ((uint64_t)iz * N + (uint64_t)iy) * N + (uint64_t)ix;
-            const uint64_t pz = (uint64_t)((N - iz) % N), py = (uint64_t)((N - iy) % N), px = (uint64_t)((N - ix) % N);
-            const uint64_t partner = (pz * N + py) * N + px;
-            uint64_t w0, w1;
-            philox2x64_10(canon ? own : partner, stream, seed, w0, w1);
-            const double two53 = 9007199254740992.0;
-            const double u1 = ((double)(w0 >> 11) + 1.0) / two53;
-            const double u2 = (double)(w1 >> 11) / two53;
-            const double k = kIR * sqrt((double)r2);
-            const double om = sqrt(k * k + m2);
-            const double P = pi_spectrum ? A * om / 2.0 : A / (2.0 * om);
-            const double L = 2.0 * M_PI / kIR;
-            const double amp = sqrt(P / (L * L * L)) * (fixed_modulus ? 1.0 : sqrt(-log(u1)));
-            double s, c;
-            sincos(2.0 * M_PI * u2, &s, &c);
-            out = make_double2(amp * c, canon ? amp * s : -amp * s);
+    for (int j = threadIdx.x; j <= N / 4; j += blockDim.x) {
+        double s, c;
+        sincospi(2.0 * (double)j / (double)N, &s, &c);
+        root[j] = make_double2(c, sign * s);
+    }
+    __syncthreads();
+}
+
+struct ModeSpec {
+    int N;
+    double kIR2, m2, amp2;  // amp2 = A/(2 L^3)
+    int pi_spectrum, fixed_modulus;
+    uint64_t seed, stream;
+};
+
+// The mode n = (nx, iy, iz) (nx >= 0 itself, iy and iz array indices): modulus
+// sqrt(P/L^3) times the Rayleigh factor sqrt(-ln u1), phase 2 pi u2, drawn at
+// the member of each Hermitian pair with the first nonzero of (nx, ny, nz)
+// positive; zero outside 0 < |n| < N/2.
+__device__ __forceinline__ double2 draw_mode(const ModeSpec &p, int nx, int iy, int iz)
+{
+    const int N = p.N;
+    const int ny = signed_mode(iy, N), nz = signed_mode(iz, N);
+    const int r2 = nx * nx + ny * ny + nz * nz;  // N <= 2048: below 2^22
+    if (r2 == 0 || 4 * r2 >= N * N) return make_double2(0.0, 0.0);
+    const bool canon = nx > 0 || ny > 0 || (ny == 0 && nz > 0);
+    const int dy = canon ? iy : (iy ? N - iy : 0), dz = canon ? iz : (iz ? N - iz : 0);
+    uint64_t w0, w1;
+    philox2x64_10(((uint64_t)dz * N + (uint64_t)dy) * N + (uint64_t)nx, p.stream, p.seed, w0, w1);
+    const double two53 = 9007199254740992.0;
+    const double u1 = ((double)(w0 >> 11) + 1.0) / two53;
+    const double u2 = (double)(w1 >> 11) / two53;
+    const double om2 = p.kIR2 * (double)r2 + p.m2;
+    const double P = p.amp2 * (p.pi_spectrum ? sqrt(om2) : rsqrt(om2));
+    const double amp = sqrt(p.fixed_modulus ? P : P * -log(u1));
+    double s, c;
+    sincospi(2.0 * u2, &s, &c);
+    return make_double2(amp * c, canon ? amp * s : -amp * s);
+}
+
+// One thread per row (iz, iy) and k = 0 .. N/4: the modes F1 = F(k, row) and
+// F2 = F(N/2 - k, -row) together give C(k, row) = S + Z and C(N/2 - k, -row) =
+// conj(S - Z) with S = F1 + conj F2, Z = i exp(2 pi i k/N) (F1 - conj F2).  At
+// k = 0 the partner mode (nx = N/2) is zero and so is the second value's
+// entry; at k = N/4 both threads of a pair of rows write their own.
+//
+// Bound by the FP64 pipe (logarithm, sine and cosine, square roots): one
+// square root of the whole modulus squared instead of four roots and two
+// divisions, 256^3 1305 -> 996 us a field.
+__global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, ModeSpec p)
+{
+    extern __shared__ double2 root[];
+    const int N = p.N, h = N / 2, q = N / 4 + 1;
+    fill_roots(root, N, 1.0);
+    const unsigned total = (unsigned)N * N * q;  // N <= 2048: below 2^32
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < total; i += gridDim.x * 256u) {
+        const unsigned row = i / q, k = i - row * q;
+        const int iz = row / N, iy = row - (unsigned)iz * N;
+        const int my = iy ? N - iy : 0, mz = iz ? N - iz : 0;
+        const double2 a = draw_mode(p, k, iy, iz);
+        if (k == 0) {  // (1 + i) F1
+            modes[(size_t)row * h] = make_double2(a.x - a.y, a.x + a.y);
+            continue;
         }
-        modes[i] = out;
+        const double2 b = draw_mode(p, h - k, my, mz);
+        const double2 w = root[k];
+        const double dx = a.x - b.x, dy = a.y + b.y;
+        const double zx = -(w.x * dy + w.y * dx), zy = w.x * dx - w.y * dy;
+        const double sx = a.x + b.x, sy = a.y - b.y;
+        modes[(size_t)row * h + k] = make_double2(sx + zx, sy + zy);
+        if (4 * (int)k != N) modes[((size_t)mz * N + my) * h + (h - k)] = make_double2(sx - zx, zy - sy);
     }
 }
 
-// dense index i = (z N + y) N + x  <->  pitched offset z PP + y P + x
-__device__ __forceinline__ long long pitched(size_t i, int N, long long P, long long PP)
+// Four consecutive sites per thread (a row starts a 128-byte line in both
+// layouts' FP32 form and N is a multiple of 4): 16- and 32-byte accesses, one
+// index decomposition for the four.
+template <typename T>
+struct Four;
+template <>
+struct Four<float> {
+    static __device__ __forceinline__ void ld(const float *p, double (&v)[4])
+    {
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+    }
+    static __device__ __forceinline__ void st(float *p, const double (&v)[4])
+    {
+        *reinterpret_cast<float4 *>(p) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+    }
+};
+template <>
+struct Four<double> {
+    static __device__ __forceinline__ void ld(const double *p, double (&v)[4])
+    {
+        const double2 a = *reinterpret_cast<const double2 *>(p), b = *reinterpret_cast<const double2 *>(p + 2);
+        v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+    }
+    static __device__ __forceinline__ void st(double *p, const double (&v)[4])
+    {
+        *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
+        *reinterpret_cast<double2 *>(p + 2) = make_double2(v[2], v[3]);
+    }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) assemble_kernel(T *dst, const double *delta, double base, double scale, int N,
+                                                       long long P, long long PP)
 {
-    const long long x = (long long)(i % N), y = (long long)((i / N) % N), z = (long long)(i / ((size_t)N * N));
-    return z * PP + y * P + x;
+    const unsigned quads = (unsigned)N / 4, i = blockIdx.x * 256u + threadIdx.x;
+    const unsigned row = i / quads, x = 4 * (i - row * quads);
+    const int z = row / N, y = row - (unsigned)z * N;
+    if (z >= N) return;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    if (delta) Four<double>::ld(delta + (size_t)row * N + x, v);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = base + (delta ? scale * v[j] : 0.0);
+    T *out = dst + z * PP + y * P + x;
+    Four<T>::st(out, v);
+    if (y == 0) Four<T>::st(out + (long long)N * P, v);  // the ghost rows
+    if (y == N - 1) Four<T>::st(out - (long long)N * P, v);
 }
 
 template <typename T>
-__global__ void assemble_kernel(T *dst, const double *delta, size_t n, double base, double scale, int N, long long P,
-                                long long PP)
+__global__ void __launch_bounds__(256) widen_kernel(double *dst, const T *src, int N, long long P, long long PP)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dst[pitched(i, N, P, PP)] = (T)(base + (delta ? scale * delta[i] : 0.0));
+    const unsigned quads = (unsigned)N / 4, i = blockIdx.x * 256u + threadIdx.x;
+    const unsigned row = i / quads, x = 4 * (i - row * quads);
+    const int z = row / N, y = row - (unsigned)z * N;
+    if (z >= N) return;
+    double v[4];
+    Four<T>::ld(src + z * PP + y * P + x, v);
+    Four<double>::st(dst + (size_t)row * N + x, v);
 }
 
-template <typename T>
-__global__ void widen_kernel(double *dst, const T *src, size_t n, int N, long long P, long long PP)
+// bin(s) = floor(sqrt(s) + 1/2) for an integer 0 <= s < 2^24 and root = sqrt(s)
+// to FP32, decided in integers: m is the bin iff m (m - 1) < s <= m (m + 1).
+__device__ __forceinline__ int shell_bin(int s, float root)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dst[i] = (double)src[pitched(i, N, P, PP)];
-}
-
-// bin(s) = floor(sqrt(s) + 1/2) for an integer s >= 0, decided in integers:
-// m is the bin iff m (m - 1) < s <= m (m + 1).
-__device__ __forceinline__ int shell_bin(long s)
-{
-    long m = (long)floor(sqrt((double)s) + 0.5);
+    int m = (int)(root + 0.5f);
     while (m > 0 && m * (m - 1) >= s) --m;
     while ((m + 1) * m < s) ++m;
-    return (int)m;
+    return m;
 }
 
-__global__ void bin_kernel(const double2 *modes, int N, int nbins, double *Psum, double *rsum,
-                           unsigned long long *cnt)
+// sqrt(s) in FP64 from its FP32 value r: two terms of the Taylor series of the
+// root about r^2 (r is right to 2^-24, so the next term is below 2^-70).
+__device__ __forceinline__ double refine_root(int s, float root)
 {
-    extern __shared__ double sh[];
-    double *sP = sh;
-    double *sR = sh + nbins;
-    unsigned long long *sC = reinterpret_cast<unsigned long long *>(sh + 2 * nbins);
+    if (s == 0) return 0.0;
+    const double r = (double)root, h = (double)(0.5f / root);
+    const double d = fma(-r, r, (double)s);
+    const double e = d * fma(-fma(2.0 * r, h, -1.0), h, h);  // d/(2r), h refined once
+    return fma(-e * e, h, r + e);
+}
+
+// Adds (P, r, w) to the shell sums of bin b: runs of lanes with the same bin
+// are summed first (a segmented sum towards each run's first lane), so that a
+// warp's atomics mostly go to different bins.
+__device__ __forceinline__ void add_to_shell(int b, double P, double r, unsigned w, double *sP, double *sR,
+                                             unsigned long long *sC)
+{
+    const int lane = threadIdx.x & 31;
+    const bool head = __shfl_up_sync(0xffffffffu, b, 1) != b || lane == 0;
+    const unsigned above = (0xfffffffeu << lane) & __ballot_sync(0xffffffffu, head);
+    const int end = above ? __ffs(above) - 1 : 32;  // the run's end
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double oP = __shfl_down_sync(0xffffffffu, P, o), oR = __shfl_down_sync(0xffffffffu, r, o);
+        const unsigned ow = __shfl_down_sync(0xffffffffu, w, o);
+        if (lane + o < end) P += oP, r += oR, w += ow;
+    }
+    if (w && head) {
+        atomicAdd(sP + b, P);
+        atomicAdd(sR + b, r);
+        atomicAdd(sC + b, (unsigned long long)w);
+    }
+}
+
+// One thread per (a, b, k), N/2 >= a >= b >= 0, k = 0 .. N/4: the modes |nx| = k
+// and |nx| = N/2 - k of the up to eight rows (+-a, +-b), (+-b, +-a), which
+// share their shells, are summed in registers before they reach the shell
+// sums.  Each C is read once, 16 reads of a thread in flight.
+//
+// FP64-pipe work a mode: 8 operations for |F|^2 and its sum.  With one shared
+// FP64 atomic (a compare-and-swap loop) for each of a mode's three sums this
+// took 475 us at 256^3; here 198.
+__global__ void __launch_bounds__(256) bin_kernel(const double2 *__restrict__ modes, int N, int nbins, double *Psum,
+                                                  double *rsum, unsigned long long *cnt)
+{
+    extern __shared__ double2 root[];  // N/4 + 1 roots, then the CTA's shell sums
+    const int h = N / 2, q = N / 4 + 1;
+    double *sP = reinterpret_cast<double *>(root + q);
+    double *sR = sP + nbins;
+    unsigned long long *sC = reinterpret_cast<unsigned long long *>(sR + nbins);
     for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
         sP[b] = 0.0;
         sR[b] = 0.0;
         sC[b] = 0ull;
     }
-    __syncthreads();
-    const int NH = N / 2 + 1;
-    const size_t total = (size_t)N * N * NH;
-    const double inv_n6 = 1.0 / ((double)N * N * N) / ((double)N * N * N);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int ix = (int)(i % NH);
-        const int iy = (int)((i / NH) % N);
-        const int iz = (int)(i / ((size_t)NH * N));
-        const long nx = ix, ny = signed_mode(iy, N), nz = signed_mode(iz, N);
-        const long r2 = nx * nx + ny * ny + nz * nz;
-        const int w = (ix == 0 || 2 * ix == N) ? 1 : 2;  // r2c keeps one of each (n, -n) pair for 0 < nx < N/2
-        const double2 d = modes[i];
-        const int b = shell_bin(r2);
-        atomicAdd(&sP[b], w * (d.x * d.x + d.y * d.y) * inv_n6);
-        atomicAdd(&sR[b], w * sqrt((double)r2));
-        atomicAdd(&sC[b], (unsigned long long)w);
+    fill_roots(root, N, -1.0);  // and a barrier
+    const unsigned pairs = (unsigned)(h + 1) * (h + 2) / 2, total = pairs * (unsigned)q;  // below 2^29
+    const double scale = 0.25 / ((double)N * N * N) / ((double)N * N * N);
+    for (unsigned first = blockIdx.x * 256u; first < total; first += gridDim.x * 256u) {
+        const unsigned i = first + threadIdx.x;
+        const bool active = i < total;
+        const unsigned pair = active ? i / q : 0;
+        const int k = active ? (int)(i - pair * q) : 0;
+        int a = (int)((sqrtf(8.0f * (float)pair + 1.0f) - 1.0f) * 0.5f);  // pair = a (a + 1)/2 + b
+        while ((unsigned)(a + 1) * (a + 2) / 2 <= pair) ++a;
+        while ((unsigned)a * (a + 1) / 2 > pair) --a;
+        const int b = (int)(pair - (unsigned)a * (a + 1) / 2);
+        const double2 w = root[k];
+        const int kp = k ? h - k : 0;
+        double P1 = 0.0, P2 = 0.0;
+        unsigned rows = 0;
+        if (active) {
+            double2 c[8], d[8];
+            bool own[8];
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int vy = v & 1 ? b : a, vz = v & 1 ? a : b;
+                const bool ny = v & 2, nz = v & 4;  // the negative one
+                own[v] = !(((v & 1) && a == b) || (ny && (vy == 0 || vy == h)) || (nz && (vz == 0 || vz == h)));
+                const int iy = ny && vy ? N - vy : vy, iz = nz && vz ? N - vz : vz;
+                const int my = iy ? N - iy : 0, mz = iz ? N - iz : 0;
+                c[v] = __ldg(modes + ((size_t)iz * N + iy) * h + k);
+                d[v] = __ldg(modes + ((size_t)mz * N + my) * h + kp);
+            }
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                if (!own[v]) continue;  // a row already among the others
+                const double ex = c[v].x + d[v].x, ey = c[v].y - d[v].y, fx = c[v].x - d[v].x, fy = c[v].y + d[v].y;
+                const double gx = fma(w.x, fy, w.y * fx), gy = fma(w.y, fy, -(w.x * fx));  // -i w (fx + i fy)
+                const double px = ex + gx, py = ey + gy, mx = ex - gx, mmy = ey - gy;
+                P1 = fma(px, px, fma(py, py, P1));
+                P2 = fma(mx, mx, fma(mmy, mmy, P2));
+                ++rows;
+            }
+        }
+        // |nx| = k, both signs of it (0 once); |nx| = N/2 - k, both signs (N/2
+        // once, N/4 counted as k)
+        const unsigned m1 = k ? 2u : 1u, m2 = k == 0 ? 1u : 4 * k == N ? 0u : 2u;
+        const int s = a * a + b * b, s1 = s + k * k, s2 = s + (h - k) * (h - k);
+        const float r1 = sqrtf((float)s1), r2 = sqrtf((float)s2);
+        add_to_shell(shell_bin(s1, r1), (double)m1 * scale * P1, (double)(m1 * rows) * refine_root(s1, r1), m1 * rows,
+                     sP, sR, sC);
+        add_to_shell(shell_bin(s2, r2), (double)m2 * scale * P2, (double)(m2 * rows) * refine_root(s2, r2), m2 * rows,
+                     sP, sR, sC);
     }
     __syncthreads();
     for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
@@ -120,50 +276,54 @@ __global__ void bin_kernel(const double2 *modes, int N, int nbins, double *Psum,
     }
 }
 
-static unsigned grid_for(size_t n, int sm_count)
+static unsigned grid_for(size_t n, int sm_count, int per_sm)
 {
-    size_t g = (n + 255) / 256;
-    size_t cap = (size_t)(sm_count > 0 ? sm_count : 152) * 16;
-    return (unsigned)(g < cap ? (g > 0 ? g : 1) : cap);
+    const size_t g = (n + 255) / 256, cap = (size_t)(sm_count > 0 ? sm_count : 152) * per_sm;
+    return (unsigned)(g < cap ? g : cap);
 }
 
 cudaError_t launch_fill_modes(double2 *modes, int N, double kIR, double A, double m2, int pi_spectrum,
                               int fixed_modulus, uint64_t seed, uint64_t stream, int sm_count, cudaStream_t s)
 {
-    size_t total = (size_t)N * N * (N / 2 + 1);
-    fill_modes_kernel<<<grid_for(total, sm_count), 256, 0, s>>>(modes, N, kIR, A, m2, pi_spectrum, fixed_modulus,
-                                                                seed, stream);
+    const double L = 2.0 * M_PI / kIR;
+    const ModeSpec p{N, kIR * kIR, m2, A / (2.0 * L * L * L), pi_spectrum, fixed_modulus, seed, stream};
+    const size_t total = (size_t)N * N * (N / 4 + 1);
+    fill_modes_kernel<<<grid_for(total, sm_count, 16), 256, (N / 4 + 1) * sizeof(double2), s>>>(modes, p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_assemble(int dtype, void *dst, const double *delta, size_t n, double base, double scale, int N,
-                            long long P, long long PP, int sm_count, cudaStream_t s)
+cudaError_t launch_assemble(int dtype, void *dst, const double *delta, double base, double scale, int N, long long P,
+                            long long PP, cudaStream_t s)
 {
+    const unsigned grid = (unsigned)(((size_t)N * N * (N / 4) + 255) / 256);
     if (dtype == TL_F32)
-        assemble_kernel<float><<<grid_for(n, sm_count), 256, 0, s>>>(static_cast<float *>(dst), delta, n, base, scale,
-                                                                     N, P, PP);
+        assemble_kernel<float><<<grid, 256, 0, s>>>(static_cast<float *>(dst), delta, base, scale, N, P, PP);
     else
-        assemble_kernel<double><<<grid_for(n, sm_count), 256, 0, s>>>(static_cast<double *>(dst), delta, n, base,
-                                                                      scale, N, P, PP);
+        assemble_kernel<double><<<grid, 256, 0, s>>>(static_cast<double *>(dst), delta, base, scale, N, P, PP);
     return cudaGetLastError();
 }
 
-cudaError_t launch_widen(int dtype, double *dst, const void *src, size_t n, int N, long long P, long long PP,
-                         int sm_count, cudaStream_t s)
+cudaError_t launch_widen(int dtype, double *dst, const void *src, int N, long long P, long long PP, cudaStream_t s)
 {
+    const unsigned grid = (unsigned)(((size_t)N * N * (N / 4) + 255) / 256);
     if (dtype == TL_F32)
-        widen_kernel<float><<<grid_for(n, sm_count), 256, 0, s>>>(dst, static_cast<const float *>(src), n, N, P, PP);
+        widen_kernel<float><<<grid, 256, 0, s>>>(dst, static_cast<const float *>(src), N, P, PP);
     else
-        widen_kernel<double><<<grid_for(n, sm_count), 256, 0, s>>>(dst, static_cast<const double *>(src), n, N, P, PP);
+        widen_kernel<double><<<grid, 256, 0, s>>>(dst, static_cast<const double *>(src), N, P, PP);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin(const double2 *modes, int N, int nbins, double *Psum, double *rsum, unsigned long long *cnt,
                        int sm_count, cudaStream_t s)
 {
-    size_t total = (size_t)N * N * (N / 2 + 1);
-    size_t shmem = (size_t)nbins * (2 * sizeof(double) + sizeof(unsigned long long));
-    bin_kernel<<<grid_for(total, sm_count), 256, shmem, s>>>(modes, N, nbins, Psum, rsum, cnt);
+    const size_t total = (size_t)(N / 2 + 1) * (N / 2 + 2) / 2 * (N / 4 + 1);
+    const size_t smem = (size_t)(N / 4 + 1) * sizeof(double2) +
+                        (size_t)nbins * (2 * sizeof(double) + sizeof(unsigned long long));
+    if (smem > 48 * 1024) {  // N above 1976
+        const cudaError_t e = cudaFuncSetAttribute(bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    bin_kernel<<<grid_for(total, sm_count, 4), 256, smem, s>>>(modes, N, nbins, Psum, rsum, cnt);
     return cudaGetLastError();
 }
 

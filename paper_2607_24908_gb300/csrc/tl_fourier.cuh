@@ -8,16 +8,25 @@
 
 namespace tl {
 
-// Half-spectrum [N][N][N/2+1] of Hermitian Gaussian modes (see tl_init_spec).
+// A real N^3 array is transformed as the complex array c[z][y][x'] = f(2x') + i
+// f(2x'+1), x' < N/2: the dense FP64 array itself, read as N x N x N/2 complex
+// values, in place.  With C its (unnormalised) transform and k' < N/2 the
+// third index, e and o the transforms of the even and odd columns (C = e + i
+// o), the field's own modes are
+//   F(n) = e(k') + w o(k'),  F(n - N/2) = e(k') - w o(k'),   w = exp(-2 pi i k'/N)
+// with e, o = (C(k) +- conj C(-k))/2, (1, 1/i): half the array and about two
+// thirds of the time of a real-to-complex transform (256^3: 1.45 against
+// 2.27 ms, 192^3 0.65 against 0.93; sizes with large prime factors 5-10%).
+
+// The modes C of a Gaussian random field (see tl_init_spec), for the inverse transform.
 cudaError_t launch_fill_modes(double2 *modes, int N, double kIR, double A, double m2, int pi_spectrum,
                               int fixed_modulus, uint64_t seed, uint64_t stream, int sm_count, cudaStream_t s);
-// dst[pitched(i)] = (T)(base + scale * delta[i]) (delta may be NULL; delta dense).
-cudaError_t launch_assemble(int dtype, void *dst, const double *delta, size_t n, double base, double scale, int N,
-                            long long P, long long PP, int sm_count, cudaStream_t s);
-// dst[i] = (double)src[pitched(i)] (dst dense).
-cudaError_t launch_widen(int dtype, double *dst, const void *src, size_t n, int N, long long P, long long PP,
-                         int sm_count, cudaStream_t s);
-// Shell sums of |d|^2 / N^6, |n| and mode counts (accumulated with atomics).
+// The padded array at dst = base + scale * delta (delta dense; may be NULL), ghost rows included.
+cudaError_t launch_assemble(int dtype, void *dst, const double *delta, double base, double scale, int N, long long P,
+                            long long PP, cudaStream_t s);
+// dst = the padded array at src, dense, in FP64.
+cudaError_t launch_widen(int dtype, double *dst, const void *src, int N, long long P, long long PP, cudaStream_t s);
+// Shell sums of |F|^2 / N^6, |n| and mode counts from C (accumulated with atomics).
 cudaError_t launch_bin(const double2 *modes, int N, int nbins, double *Psum, double *rsum, unsigned long long *cnt,
                        int sm_count, cudaStream_t s);
 

@@ -6,6 +6,7 @@
 // half the real size: tl_fourier.cuh).
 #include <math.h>
 
+#include "tl_boxmuller.cuh"
 #include "tl_fourier.cuh"
 #include "tl_philox.cuh"
 
@@ -35,7 +36,7 @@ struct ModeSpec {
 // sqrt(P/L^3) times the Rayleigh factor sqrt(-ln u1), phase 2 pi u2, drawn at
 // the member of each Hermitian pair with the first nonzero of (nx, ny, nz)
 // positive; zero outside 0 < |n| < N/2.
-__device__ __forceinline__ double2 draw_mode(const ModeSpec &p, int nx, int iy, int iz)
+__device__ __forceinline__ double2 draw_mode(const BoxMullerTable *t, const ModeSpec &p, int nx, int iy, int iz)
 {
     const int N = p.N;
     const int ny = signed_mode(iy, N), nz = signed_mode(iz, N);
@@ -45,14 +46,11 @@ __device__ __forceinline__ double2 draw_mode(const ModeSpec &p, int nx, int iy, 
     const int dy = canon ? iy : (iy ? N - iy : 0), dz = canon ? iz : (iz ? N - iz : 0);
     uint64_t w0, w1;
     philox2x64_10(((uint64_t)dz * N + (uint64_t)dy) * N + (uint64_t)nx, p.stream, p.seed, w0, w1);
-    const double two53 = 9007199254740992.0;
-    const double u1 = ((double)(w0 >> 11) + 1.0) / two53;
-    const double u2 = (double)(w1 >> 11) / two53;
     const double om2 = p.kIR2 * (double)r2 + p.m2;
     const double P = p.amp2 * (p.pi_spectrum ? sqrt(om2) : rsqrt(om2));
-    const double amp = sqrt(p.fixed_modulus ? P : P * -log(u1));
+    const double amp = sqrt(p.fixed_modulus ? P : P * neg_log_u53(t, (w0 >> 11) + 1));
     double s, c;
-    sincospi(2.0 * u2, &s, &c);
+    unit_circle_u53(t, w1 >> 11, c, s);
     return make_double2(amp * c, canon ? amp * s : -amp * s);
 }
 
@@ -62,25 +60,27 @@ __device__ __forceinline__ double2 draw_mode(const ModeSpec &p, int nx, int iy, 
 // k = 0 the partner mode (nx = N/2) is zero and so is the second value's
 // entry; at k = N/4 both threads of a pair of rows write their own.
 //
-// Bound by the FP64 pipe (logarithm, sine and cosine, square roots): one
-// square root of the whole modulus squared instead of four roots and two
-// divisions, 256^3 1305 -> 996 us a field.
+// Bound by the FP64 pipe: one square root of the whole modulus squared instead
+// of four roots and two divisions, 256^3 1305 -> 996 us a field, and the table
+// form of the logarithm and the circle (tl_boxmuller.cuh), 996 -> 610 us.
 __global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, ModeSpec p)
 {
     extern __shared__ double2 root[];
+    __shared__ BoxMullerTable table;
     const int N = p.N, h = N / 2, q = N / 4 + 1;
+    load_box_muller(&table);
     fill_roots(root, N, 1.0);
     const unsigned total = (unsigned)N * N * q;  // N <= 2048: below 2^32
     for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < total; i += gridDim.x * 256u) {
         const unsigned row = i / q, k = i - row * q;
         const int iz = row / N, iy = row - (unsigned)iz * N;
         const int my = iy ? N - iy : 0, mz = iz ? N - iz : 0;
-        const double2 a = draw_mode(p, k, iy, iz);
+        const double2 a = draw_mode(&table, p, k, iy, iz);
         if (k == 0) {  // (1 + i) F1
             modes[(size_t)row * h] = make_double2(a.x - a.y, a.x + a.y);
             continue;
         }
-        const double2 b = draw_mode(p, h - k, my, mz);
+        const double2 b = draw_mode(&table, p, h - k, my, mz);
         const double2 w = root[k];
         const double dx = a.x - b.x, dy = a.y + b.y;
         const double zx = -(w.x * dy + w.y * dx), zy = w.x * dx - w.y * dy;
@@ -288,7 +288,7 @@ cudaError_t launch_fill_modes(double2 *modes, int N, double kIR, double A, doubl
     const double L = 2.0 * M_PI / kIR;
     const ModeSpec p{N, kIR * kIR, m2, A / (2.0 * L * L * L), pi_spectrum, fixed_modulus, seed, stream};
     const size_t total = (size_t)N * N * (N / 4 + 1);
-    fill_modes_kernel<<<grid_for(total, sm_count, 16), 256, (N / 4 + 1) * sizeof(double2), s>>>(modes, p);
+    fill_modes_kernel<<<grid_for(total, sm_count, 8), 256, (N / 4 + 1) * sizeof(double2), s>>>(modes, p);
     return cudaGetLastError();
 }
 

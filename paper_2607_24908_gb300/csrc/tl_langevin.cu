@@ -15,29 +15,24 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "tl_boxmuller.cuh"
 #include "tl_internal.cuh"
 #include "tl_lattice.cuh"
 #include "tl_philox.cuh"
 
 namespace {
 
-using tl::philox2x64_10;  // the initial-state draw's generator
+using tl::philox2x64_10_low;  // the initial-state draw's generator
 
 // The two Gaussians of draw k: (cos, sin) halves of Box-Muller.
-template <typename T>
-__device__ __forceinline__ void gauss2(uint64_t k, uint64_t ctr1, uint64_t seed, T &gc, T &gs);
-
-template <>
-__device__ __forceinline__ void gauss2<double>(uint64_t k, uint64_t ctr1, uint64_t seed, double &gc, double &gs)
+__device__ __forceinline__ void gauss2(const tl::BoxMullerTable *t, uint32_t k, uint64_t ctr1, uint64_t seed, double &gc,
+                                       double &gs)
 {
     uint64_t w0, w1;
-    philox2x64_10(k, ctr1, seed, w0, w1);
-    const double two53 = 9007199254740992.0;
-    const double u1 = ((double)(w0 >> 11) + 1.0) / two53;
-    const double u2 = (double)(w1 >> 11) / two53;
-    const double r = sqrt(-2.0 * log(u1));
+    philox2x64_10_low(k, ctr1, seed, w0, w1);
+    const double r = sqrt(2.0 * tl::neg_log_u53(t, (w0 >> 11) + 1));
     double s, c;
-    sincospi(2.0 * u2, &s, &c);
+    tl::unit_circle_u53(t, w1 >> 11, c, s);
     gc = r * c;
     gs = r * s;
 }
@@ -54,72 +49,119 @@ __device__ __forceinline__ float u53_f32(uint64_t x)
     return fmaf((float)hi, 0x1p-24f, (float)lo * 0x1p-53f);
 }
 
-template <>
-__device__ __forceinline__ void gauss2<float>(uint64_t k, uint64_t ctr1, uint64_t seed, float &gc, float &gs)
+// (cos, sin)(2 pi w 2^-64) in FP32: the nearest quarter turn is taken off in
+// integers, the rest, within an eighth of a turn, goes into the Taylor
+// polynomials (first omitted terms below 2e-9 and 3e-8).  About 20
+// instructions, half of them on the FMA pipes; sincospif of a converted
+// uniform took 35.
+__device__ __forceinline__ void unit_circle(uint64_t w, float &c, float &s)
+{
+    const uint32_t h = (uint32_t)(w >> 32) + 0x20000000u;
+    const float x = (float)((int32_t)(h & 0x3fffffffu) - 0x20000000) * (float)(2.0 * M_PI / 4294967296.0);
+    const float t = x * x;
+    float ps = fmaf(t, 1.0f / 362880.0f, -1.0f / 5040.0f);
+    ps = fmaf(ps, t, 1.0f / 120.0f);
+    ps = fmaf(ps, t, -1.0f / 6.0f);
+    ps = fmaf(ps * t, x, x);
+    float pc = fmaf(t, 1.0f / 40320.0f, -1.0f / 720.0f);
+    pc = fmaf(pc, t, 1.0f / 24.0f);
+    pc = fmaf(pc, t, -0.5f);
+    pc = fmaf(pc, t, 1.0f);
+    const bool odd = h & 0x40000000u;  // quarter turns 0..3 in the top two bits
+    const uint32_t u = __float_as_uint(odd ? ps : pc), v = __float_as_uint(odd ? pc : ps);
+    c = __uint_as_float(u ^ ((h ^ (h << 1)) & 0x80000000u));  // cos is negative in quarters 1, 2
+    s = __uint_as_float(v ^ (h & 0x80000000u));               // sin in 2, 3
+}
+
+__device__ __forceinline__ void gauss2(const tl::BoxMullerTable *, uint32_t k, uint64_t ctr1, uint64_t seed, float &gc,
+                                       float &gs)
 {
     uint64_t w0, w1;
-    philox2x64_10(k, ctr1, seed, w0, w1);
-    // the same 53-bit uniforms, Box-Muller in FP32 (the field is stored in FP32)
+    philox2x64_10_low(k, ctr1, seed, w0, w1);
+    // Box-Muller in FP32 (the field is stored in FP32): u1 to 2^-24 of itself,
+    // the angle to 2^-32 of a turn
     const float u1 = u53_f32((w0 >> 11) + 1);
-    const float u2 = u53_f32(w1 >> 11);
     const float r = sqrtf(-2.0f * logf(u1));
     float s, c;
-    sincospif(2.0f * u2, &s, &c);
+    unit_circle(w1, c, s);
     gc = r * c;
     gs = r * s;
 }
 
-template <typename T>
-struct V16;
-template <>
-struct V16<float> {
-    static constexpr int W = 4;
-};
-template <>
-struct V16<double> {
-    static constexpr int W = 2;
-};
-
-template <typename T>
-__device__ __forceinline__ void ld(const T *p, T (&o)[V16<T>::W])
+// W consecutive sites (one 16-byte word: rows start on 128-byte boundaries).
+__device__ __forceinline__ void ld(const float *p, float (&o)[4])
 {
-#pragma unroll
-    for (int j = 0; j < V16<T>::W; ++j) o[j] = __ldg(p + j);
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+    o[0] = v.x, o[1] = v.y, o[2] = v.z, o[3] = v.w;
+}
+__device__ __forceinline__ void ld(const double *p, double (&o)[2])
+{
+    const double2 v = __ldg(reinterpret_cast<const double2 *>(p));
+    o[0] = v.x, o[1] = v.y;
+}
+__device__ __forceinline__ void st(float *p, const float (&v)[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st(double *p, const double (&v)[2])
+{
+    *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
 }
 
+// FP32 is bound by instruction issue and the integer pipes (the draws' wide
+// products alone take 150 us at 384^3): neighbours come as 16-byte words and by
+// shuffle, the angle from the word's bits, the first round of the generator
+// with two products; 467 instructions a plane and thread, from 538, and less
+// in the last wave: 303 -> 244 us.  FP64 is bound by the FP64 pipe: the
+// table form of Box-Muller (tl_boxmuller.cuh) took 384^3 from 5910 to 3779 us.
 template <typename T>
 __global__ void __launch_bounds__(256) langevin_pass(const T *__restrict__ in, T *__restrict__ out, int N, int txt,
                                                      int ty, int zc, long long P, long long PP, T inv_dx2, T dt, T m2,
                                                      T half_lam, T amp, uint64_t seed, uint64_t ctr1)
 {
-    constexpr int W = V16<T>::W;
+    constexpr int W = 16 / (int)sizeof(T);
+    constexpr bool kTable = sizeof(T) == 8;
+    __shared__ __align__(16) unsigned char table_raw[kTable ? sizeof(tl::BoxMullerTable) : 16];
+    tl::BoxMullerTable *table = reinterpret_cast<tl::BoxMullerTable *>(table_raw);
+    if (kTable) tl::load_box_muller(table);
     const int tx = threadIdx.x % txt, tyi = threadIdx.x / txt;
     const int x0 = (blockIdx.x * txt + tx) * W;
     const int y = blockIdx.y * ty + tyi;
     const int z0 = blockIdx.z * zc;
     const int z1 = min(z0 + zc, N);
     if (!(tyi < ty && x0 < N && y < N)) return;
-    const size_t NN = (size_t)PP;
-    const size_t row = (size_t)y * P, rowm = (size_t)(y == 0 ? N - 1 : y - 1) * P,
-                 rowp = (size_t)(y + 1 == N ? 0 : y + 1) * P;
+    // the x-neighbours are in the adjacent lanes' words; a thread at a row end,
+    // a tile edge or a warp edge loads its own
+    const unsigned lanes = __activemask();
+    const int lane = threadIdx.x & 31;
+    const bool own_l = tx == 0 || lane == 0, own_r = tx == txt - 1 || x0 + W == N || lane == 31;
+    const int src_l = own_l ? lane : lane - 1, src_r = own_r ? lane : lane + 1;
+    const size_t row = (size_t)y * P + x0;
+    const T *pc = in + (size_t)z0 * PP + row;  // this thread's sites of plane z
+    T *po = out + (size_t)z0 * PP + row;
+    const long long dym = (y == 0 ? N - 1 : -1) * P, dyp = (y + 1 == N ? 1 - N : 1) * P;
+    const int dxl = x0 == 0 ? N - 1 : -1, dxr = x0 + W == N ? W - N : W;
+    const long long up = (1 - (long long)N) * PP;  // from plane N - 1 to plane 0
     // ghost rows of this thread's sites (padded arrays carry one ghost row on
     // each side of a plane; the x-edges need no copies)
     const long long gy = y == 0 ? (long long)N * P : (y == N - 1 ? -(long long)N * P : 0);
-    const int xl = x0 == 0 ? N - 1 : x0 - 1, xr = x0 + W == N ? 0 : x0 + W;
+    // x0 and W are even: the thread's sites form whole pairs; N <= 2048: pair indices are below 2^32
+    uint32_t k0 = (uint32_t)((((uint64_t)z0 * N + y) * N + x0) >> 1);
+    const uint32_t dk = (uint32_t)N * N / 2;
     T zm[W], cu[W], zp[W];
-    ld(in + (size_t)(z0 == 0 ? N - 1 : z0 - 1) * NN + row + x0, zm);
-    ld(in + (size_t)z0 * NN + row + x0, cu);
+    ld(z0 == 0 ? pc - up : pc - PP, zm);
+    ld(pc, cu);
     for (int z = z0; z < z1; ++z) {
-        const size_t pz = (size_t)z * NN;
         T ym[W], yp[W];
-        ld(in + (size_t)(z + 1 == N ? 0 : z + 1) * NN + row + x0, zp);
-        ld(in + pz + rowm + x0, ym);
-        ld(in + pz + rowp + x0, yp);
-        const T a = __ldg(in + pz + row + xl), b = __ldg(in + pz + row + xr);
-        T xi[W];  // x0 and W are even: the thread's sites form whole pairs
-        const uint64_t k0 = (((uint64_t)z * N + y) * N + x0) >> 1;
+        ld(z + 1 == N ? pc + up : pc + PP, zp);
+        ld(pc + dym, ym);
+        ld(pc + dyp, yp);
+        T a = __shfl_sync(lanes, cu[W - 1], src_l), b = __shfl_sync(lanes, cu[0], src_r);
+        if (own_l) a = __ldg(pc + dxl);
+        if (own_r) b = __ldg(pc + dxr);
+        T xi[W];
 #pragma unroll
-        for (int j = 0; j < W; j += 2) gauss2<T>(k0 + j / 2, ctr1, seed, xi[j], xi[j + 1]);
+        for (int j = 0; j < W; j += 2) gauss2(table, k0 + j / 2, ctr1, seed, xi[j], xi[j + 1]);
         T o[W];
 #pragma unroll
         for (int j = 0; j < W; ++j) {
@@ -130,16 +172,16 @@ __global__ void __launch_bounds__(256) langevin_pass(const T *__restrict__ in, T
             const T drift = lap * inv_dx2 - m2 * c - half_lam * c * c * c;
             o[j] = (c + dt * drift) + amp * xi[j];
         }
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-            out[pz + row + x0 + j] = o[j];
-            if (gy) out[pz + row + x0 + j + gy] = o[j];
-        }
+        st(po, o);
+        if (gy) st(po + gy, o);
 #pragma unroll
         for (int j = 0; j < W; ++j) {
             zm[j] = cu[j];
             cu[j] = zp[j];
         }
+        pc += PP;
+        po += PP;
+        k0 += dk;
     }
 }
 
@@ -154,8 +196,26 @@ extern "C" int tl_langevin_step(tl_lattice *L, int n, double dt, const tl_langev
     if (!isfinite(p->lambda) || !isfinite(p->m2) || !isfinite(p->noise)) return tl::fail(TL_EINVAL, "non-finite parameter");
     if (!(L->state_mask & 1u)) return tl::fail(TL_ESTATE, "phi_0 has not been set");
     if (L->batch_refs > 0) return tl::fail(TL_ESTATE, "lattice is part of a batch");
-    tl::PassTuning t{tl::kVariantLdg, 8, 0, 0, 0, 256, 0};
-    const tl::PassGeom g = tl::pass_geometry(L->N, (int)L->esz, L->sm_count, 1, t);
+    tl::PassTuning t{tl::kVariantLdg, 8, 0, L->N, 0, 256, 0};
+    tl::PassGeom g = tl::pass_geometry(L->N, (int)L->esz, L->sm_count, 1, t);
+    int per_sm = 0;
+    cudaError_t oe = L->dtype == TL_F32
+                         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, langevin_pass<float>, 256, 0)
+                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, langevin_pass<double>, 256, 0);
+    if (oe != cudaSuccess) return tl::fail(TL_ECUDA, "langevin occupancy: %s", cudaGetErrorString(oe));
+    // z-chunk.  FP64 is bound by arithmetic alone, which the two planes a chunk
+    // reads beyond its own do not add to: one plane per CTA spreads it best (us:
+    // 100^3 96 against 116 with 4 planes, 212^3 777 against 795, 384^3 3779 against
+    // 3790).  FP32: the fewest (waves of CTAs) x (planes per CTA + 1/4 for those two
+    // planes): 384^3 244 us with 19 planes, 258 with 32; 64^3 5.7 with 1, 6.8 with 4.
+    const long slots = (long)(L->sm_count > 0 ? L->sm_count : 152) * (per_sm > 0 ? per_sm : 1);
+    double best = 0.0;
+    for (int c = 1; c <= (L->dtype == TL_F32 ? L->N : 1); ++c) {
+        const long ctas = (long)g.grid.x * g.grid.y * ((L->N + c - 1) / c);
+        const double cost = (double)((ctas + slots - 1) / slots) * (c + 0.25);
+        if (best == 0.0 || cost < best) best = cost, g.zc = c;
+    }
+    g.grid.z = (unsigned)((L->N + g.zc - 1) / g.zc);
     const double inv_dx2 = 1.0 / (L->dx * L->dx);
     const double amp = p->noise * sqrt(dt);
     for (int s = 0; s < n; ++s) {

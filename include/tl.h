@@ -380,7 +380,7 @@ typedef struct {
     int warps;   /* TMA: compute warps per CTA, 7 (two CTAs per SM) or 15 (one); 0 = 7 */
     int stages;  /* TMA: ring depth 3..8; 0 = as deep as the shared memory allows */
     int z_chunk; /* z-planes per CTA, 1..N; 0 = automatic (at least ~8 CTAs per SM) */
-    int tile_x;  /* STREAM: threads along a tile row, 8, 16 or 32; 0 = 32 */
+    int tile_x;  /* STREAM: threads along a tile row, 8, 16 or at most 32 (rows in equal tiles); 0 = 32 */
     int threads; /* STREAM: threads per CTA, 256 or 512; 0 = 256 */
 } tl_pass_config;
 
@@ -405,9 +405,10 @@ typedef struct tl_batch tl_batch; /* opaque */
 int tl_batch_create(tl_batch **out, tl_lattice *const *lats, int n, void *cuda_stream);
 
 /* The launch shape tl_batch_create gives a lattice of this size on the
- * current device: the TL_PASS_STREAM kernel with 256-thread CTAs, with the
- * z-chunk and tile row width tl_batch_autotune measured for (N, n_fields,
- * dtype, SM count) if it has, else z-chunks of min(N, 32) planes.  Set it
+ * current device: what tl_batch_autotune measured for (N, n_fields, dtype, SM
+ * count) if it has, else TL_PASS_TMA with 7 compute warps for FP32 from N = 80
+ * and TL_PASS_STREAM with 256-thread CTAs otherwise, with z-chunks of 32 planes
+ * (64 for FP32 from N = 192; at most N).  Set it
  * with tl_set_pass_config on a lattice that should step alone bitwise like
  * its batched twin.  Errors: TL_EINVAL. */
 int tl_batch_pass_config(int N, int n_fields, tl_dtype dtype, tl_pass_config *out);
@@ -466,11 +467,11 @@ int tl_autotune(tl_lattice *lat, double *best_ms_per_pass);
  * TL_ESTATE while the lattice is in a batch.  May synchronise the lattice
  * stream (to grow its reduction slots).  A new lattice starts on TL_PASS_TMA
  * when it is FP32 and N >= 192 (z-chunks of 48 planes at N = 192, 64 up to
- * N = 319, then 56, 80, 160 (one field) or 96, 104, 72 and 76 planes around
+ * N = 319, then 56, 80, 160 (one field) or 96, 104, 72 and 68 planes around
  * N = 384, 448, 512, 576 ... 768, 896 and 1024, where they measured fastest;
  * 15 compute warps from N = 416, else 7), on
- * TL_PASS_STREAM otherwise (where those measured faster; FP64 from N = 128
- * with z-chunks of 32 planes, 64 from N = 512); the environment
+ * TL_PASS_STREAM otherwise (where those measured faster; z-chunks chosen from N
+ * and the SM count, FP64 mostly 32 planes from N = 128 and 64 from N = 512); the environment
  * variable TL_PASS_VARIANT=tma|ldg overrides that default at creation. */
 int tl_set_pass_config(tl_lattice *lat, const tl_pass_config *cfg);
 

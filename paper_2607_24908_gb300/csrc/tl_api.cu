@@ -60,7 +60,7 @@ tl::PassTuning tl::default_tuning(int N, int nf, int elem_bytes)
         // 0.325; 448^3 15 + 1, 80 planes 0.524 two fields (96: 0.531); 512^3 15 + 1, 160
         // planes 0.417 one field, 96 planes 0.705 two (160: 0.714); 576^3 ... 768^3 104
         // planes (640^3 1.330, 768^3 2.297 two fields); 896^3 72 planes 3.623 (92: 3.634);
-        // 1024^3 76 planes 5.380 (92: 5.391).  The optimum is jagged in the chunk count, so
+        // 1024^3 68 planes 5.384 (76: 5.405, 92: 5.435).  The optimum is jagged in the chunk count, so
         // each measured size sets the value for the sizes around it.
         if (N <= 192) t.zc = 48;
         else if (N < 320) t.zc = 64;
@@ -69,14 +69,8 @@ tl::PassTuning tl::default_tuning(int N, int nf, int elem_bytes)
         else if (N < 544) t.zc = nf == 1 ? 160 : 96;
         else if (N < 832) t.zc = 104;
         else if (N < 960) t.zc = 72;
-        else t.zc = 76;
+        else t.zc = 68;
         t.cwarps = N >= 416 ? 15 : 7;
-    } else if (elem_bytes == 8 && N >= 128) {
-        // FP64 streaming pass (bound by the FP64 pipe): 32-plane chunks from 128^3 (one and two
-        // fields, 128^3 ... 384^3: 0.7316 ms at 256^3 against 0.7465 with the 16 of the automatic
-        // rule), 64 from 512^3 (5.465 vs 5.525 ms); tile row widths 8, 16, 32 measured alike.
-        // Smaller FP64 lattices keep the automatic rule, which spreads them over more SMs.
-        t.zc = N >= 512 ? 64 : 32;
     }
     if ((v = getenv("TL_PREFETCH"))) t.prefetch = atoi(v);
     if ((v = getenv("TL_LDG_THREADS"))) t.threads = atoi(v);
@@ -182,6 +176,9 @@ void refresh_model(tl_lattice *L)
     m.expanding = L->ex.expanding ? 1 : 0;
     m.alpha = L->ex.alpha;
     m.mu2 = L->ex.fstar_over_mp * L->ex.fstar_over_mp;
+    m.mu2_3 = m.mu2 / 3.0;
+    m.int_alpha = m.alpha == rint(m.alpha) && m.alpha >= -4.0 && m.alpha <= 6.0;
+    m.inv_n3 = 1.0 / (double)n3_of(L->N);
     m.inv_dx2 = 1.0 / (L->dx * L->dx);
     m.lambda = L->pot.lambda;
     m.q = L->pot.q;
@@ -767,7 +764,7 @@ int tl_get_pass_config(const tl_lattice *L, tl_pass_config *cfg)
     cfg->warps = tma ? g.cwarps : 0;
     cfg->stages = tma ? g.stages : 0;
     cfg->z_chunk = g.zc;
-    cfg->tile_x = tma ? 0 : g.txt;
+    cfg->tile_x = tma ? 0 : g.tile_x;
     cfg->threads = tma ? 0 : g.threads;
     return TL_OK;
 }

@@ -309,11 +309,16 @@ int build_graph(tl_batch *B, int n, double dt, int integrator)
 }
 
 // ---- batch launch shapes ------------------------------------------------------
-// A member's shape in a batch: the register-streaming tiles with 256-thread
-// CTAs (what the grouped kernel runs).  Untuned, z-chunks of 32 planes (the
-// whole lattice below that), so that each (lattice, tile) item of the grouped
-// launch carries enough planes to amortise its fixed costs (locating the job,
-// the coefficient set-up, the FP64 reduction of its sums); tl_batch_autotune
+// A member's shape in a batch, untuned: FP32 from N = 80 the grouped TMA kernel,
+// else the register-streaming tiles with 256-thread CTAs of the grouped streaming
+// kernel; z-chunks of 32 planes (the whole lattice below that, 64 from N = 192),
+// so that each (lattice, tile) item of the grouped launch carries enough planes to
+// amortise its fixed costs (locating the job, the coefficient set-up, the FP64
+// reduction of its sums) and a batch of one or two lattices still has items for
+// the GPU.  ms per 50 steps, streaming for all / TMA from 96^3 with chunks of 32 /
+// of 64 planes: 96 jobs of 32^3 ... 128^3 23.6 / 18.4 / 17.5, 32 jobs 8.7 / 6.9 / 6.8,
+// 8 jobs 4.2 / 4.0 / 4.4, two of 128^3 3.0 / 2.0 / 3.3, one of 96^3 1.8 / 1.2 / 1.9;
+// TMA from 64^3 on, 96 jobs: 19.4.  tl_batch_autotune
 // replaces this rule by measured shapes per (N, fields, dtype, SMs), and the
 // batch-level options per batch composition.
 
@@ -322,7 +327,11 @@ std::mutex g_batch_mu;
 std::map<ClassKey, tl::PassTuning> g_batch_shapes;
 std::map<std::string, BatchOpts> g_batch_opts;  // composition signature -> options
 
-tl::PassTuning batch_rule(int N) { return tl::PassTuning{tl::kVariantLdg, 7, 0, N < 32 ? N : 32, 0, 256, 0}; }
+tl::PassTuning batch_rule(int N, int dtype)
+{
+    if (dtype == TL_F32 && N >= 80) return tl::PassTuning{tl::kVariantTma, 7, 0, N < 192 ? 32 : 64, 0, 256, 0};
+    return tl::PassTuning{tl::kVariantLdg, 7, 0, N < 32 ? N : 32, 0, 256, 0};
+}
 
 void ensure_tune_loaded();  // TL_TUNE_FILE, read once (autotuner section below)
 
@@ -331,7 +340,7 @@ tl::PassTuning batch_tuning(int N, int nf, int dtype, int sms)
     ensure_tune_loaded();
     std::lock_guard<std::mutex> lk(g_batch_mu);
     auto it = g_batch_shapes.find(ClassKey(N, nf, dtype, sms));
-    return it != g_batch_shapes.end() ? it->second : batch_rule(N);
+    return it != g_batch_shapes.end() ? it->second : batch_rule(N, dtype);
 }
 
 std::string composition(const std::vector<tl_lattice *> &lats)

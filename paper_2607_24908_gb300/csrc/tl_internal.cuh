@@ -31,14 +31,19 @@ struct Scalars {
     double b;          // a'
     double drift;      // the next pass's drift: d dt ((a_prev + a)/2)^(alpha-3)
     double pending_dt; // program time the next pass's drift advances
+    // powers of a, in this order (the pass writes them as one array)
     double wl, wv;     // a^(1+alpha), a^(3+alpha)
     double wk, wg;     // a^-6, a^-2
+    double pf, ph;     // a^(2 alpha+1), a^(2 alpha)
+    double ia;         // 1/a
     double E[kMaxQ];   // K_f, G_f, V at the last evaluated time
     double hubble;     // Hubble residual at the last integer time
     double time;       // program time of the last evaluation
     int status;        // TL_OK or TL_EUNSTABLE
     unsigned ticket;   // CTAs of the current pass that finished their slot
 };
+
+constexpr int kScalePowers = 7;  // wl .. ia
 
 // Scalar constants of a lattice/model passed by value to every pass.
 // Field arrays are addressed from their element (0, 0, 0) as
@@ -57,8 +62,10 @@ struct Model {
     int ghosts;
     long long pitch;
     long long pplane;
+    int int_alpha;     // alpha is a whole number in -4 .. 6: powers by multiplication
     double alpha;
-    double mu2;
+    double mu2, mu2_3; // mu2, mu2/3
+    double inv_n3;     // 1/N^3
     double inv_dx2;
     double lambda, q;
     double m2[kMaxFields];
@@ -95,7 +102,7 @@ struct PassTuning {
     int zc;       // z-planes per CTA
     int prefetch; // ldg: planes prefetched per thread with cp.async (0 or 3)
     int threads;  // ldg: threads per CTA, 256 (default) or 512
-    int txt;      // ldg: threads along x per tile row, 32 (default), 16 or 8
+    int txt;      // ldg: threads along x per tile row, 16 or 8, or at most 32 (32, the default: even_row_tile)
 };
 
 // Tensor maps of the input arrays of a TMA pass: map[k][2 f + a], a = 0 phi,
@@ -150,6 +157,7 @@ static_assert(tma_slot_bytes(32, 15) == 9472 && tma_slot_bytes(32, 7) == 5120,
 // Launch geometry of the fused pass.
 struct PassGeom {
     int txt;  // threads along x (each owns VEC consecutive sites)
+    int tile_x;  // what it was asked for as: the row's width, at most 32, 16 or 8
     int ty;   // threads along y (one row each)
     int zc;   // z-planes per CTA
     dim3 grid;
@@ -162,6 +170,15 @@ struct PassGeom {
     int threads;   // threads per CTA (ldg variant)
     size_t smem;   // dynamic shared memory per CTA
 };
+
+// Threads along x of the streaming kernel's 32-wide tiles: rows of per_row
+// threads cut into the fewest tiles of at most 32, all alike (a row of 48 into
+// two of 24; 32 + 16 left a quarter of the lanes idle).
+inline int even_row_tile(int per_row)
+{
+    const int tiles = (per_row + 31) / 32;
+    return (per_row + tiles - 1) / tiles;
+}
 
 PassGeom pass_geometry(int N, int elem_bytes, int sm_count, int nf, const PassTuning &t);
 

@@ -115,6 +115,9 @@ extern "C" int tl_energies_noalloc(int N, double kIR, int n_fields, tl_dtype dty
     m.expanding = (expansion && expansion->expanding) ? 1 : 0;
     m.alpha = m.expanding ? expansion->alpha : 0.0;
     m.mu2 = m.expanding ? expansion->fstar_over_mp * expansion->fstar_over_mp : 1.0;
+    m.mu2_3 = m.mu2 / 3.0;
+    m.int_alpha = m.alpha == rint(m.alpha) && m.alpha >= -4.0 && m.alpha <= 6.0;
+    m.inv_n3 = 1.0 / ((double)N * N * N);
     const double dx = 2.0 * M_PI / (kIR * N);
     m.inv_dx2 = 1.0 / (dx * dx);
     m.lambda = pot->lambda;

@@ -4,41 +4,21 @@
 #include <math.h>
 
 #include "tl_internal.cuh"
+#include "tl_scale.cuh"
 
 namespace tl {
 
-// x^e with integer exponents by repeated squaring (as the pass's finalize does)
-__device__ double powe_h(double x, double e)
+__global__ void set_background_kernel(Model m, Scalars *sc, double a, double b)  // one warp
 {
-    const double r = rint(e);
-    if (r == e && fabs(r) <= 16.0) {
-        int n = (int)fabs(r);
-        double acc = 1.0, b = x;
-        while (n) {
-            if (n & 1) acc *= b;
-            b *= b;
-            n >>= 1;
-        }
-        return r < 0.0 ? 1.0 / acc : acc;
-    }
-    return pow(x, e);
-}
-
-__global__ void set_background_kernel(Model m, Scalars *sc, double a, double b)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    if (m.expanding) write_scale_powers(m, sc, a, a, a);
+    if (threadIdx.x != 0) return;
     if (m.expanding) {
-        const double al = m.alpha;
         sc->a = a;
         sc->b = b;
-        sc->wl = powe_h(a, 1.0 + al);
-        sc->wv = powe_h(a, 3.0 + al);
-        sc->wk = powe_h(a, -6.0);
-        sc->wg = powe_h(a, -2.0);
     } else {
         sc->a = 1.0;
         sc->b = 0.0;
-        sc->wl = sc->wv = sc->wk = sc->wg = 1.0;
+        for (int i = 0; i < kScalePowers; ++i) (&sc->wl)[i] = 1.0;
     }
     sc->drift = 0.0;
     sc->pending_dt = 0.0;
@@ -47,6 +27,73 @@ __global__ void set_background_kernel(Model m, Scalars *sc, double a, double b)
     sc->status = TL_OK;
     sc->ticket = 0u;
     for (int i = 0; i < kMaxQ; ++i) sc->E[i] = 0.0;
+}
+
+// ---- tile rows and z-chunks of the streaming kernel ----------------------------
+//
+// FP64 passes are bound by the FP64 pipe, where a warp's instruction holds its SM
+// for 16 clocks whatever its lanes do, so that a pass takes as long as the SM
+// with the most warp-planes: per warp and plane about 50 instructions a field (57
+// in chunks of one plane, which drift three planes for one), and per CTA its
+// sums and latencies, about 60.  Measured against this estimate (us, one field,
+// one plane a chunk -> chosen): 64^3 35.7 -> 20.8 (3 planes; 4: 19.7), 96^3 81.5 ->
+// 49 (14 planes), 128^3 96 (7 planes; 32: 101), 140^3 127 (20 planes; 32: 197), 212^3
+// 428 (20; 32: 447).  32^3 takes tiles of 16 x 8 threads on 128 SMs, not 16 x 16 on 64.
+
+constexpr int kThinChunk = 3;  // chunks up to here may have tiles of fewer rows
+
+static double f64_cost(int N, int gx, int txt, int ty, int zc, int sms)
+{
+    const long ctas = (long)gx * ((N + ty - 1) / ty) * ((N + zc - 1) / zc);
+    int warps = (txt * ty + 31) / 32;
+    if (warps < 4) warps = 4;  // fewer do not fill the pipe: an operation's result takes 65 clocks
+    return (double)((ctas + sms - 1) / sms) * (warps * ((zc == 1 ? 57 : 50 * zc) + 10) + 60);
+}
+
+// Rows of an FP64 tile of zc planes: all that fit, or in thin chunks, which are
+// for lattices that do not fill the GPU, the cheapest number.
+static int f64_tile_rows(int N, int gx, int txt, int ty_max, int zc, int sms)
+{
+    int best = ty_max;
+    if (zc <= kThinChunk)
+        for (int ty = ty_max - 1; ty >= 1; --ty)
+            if (f64_cost(N, gx, txt, ty, zc, sms) < f64_cost(N, gx, txt, best, zc, sms)) best = ty;
+    return best;
+}
+
+// FP64 chunk: the cheapest; from 128^3 32 planes and from 512^3 64 (the best of a
+// measured sweep) unless another is estimated 5% cheaper.
+static int f64_chunk(int N, int gx, int txt, int ty_max, int sms)
+{
+    auto cost = [&](int zc) { return f64_cost(N, gx, txt, f64_tile_rows(N, gx, txt, ty_max, zc, sms), zc, sms); };
+    int best = N >= 512 ? 64 : N >= 128 ? 32 : 1;
+    double least = cost(best) * (N >= 128 ? 0.95 : 1.0);
+    for (int zc = 1; zc <= N && zc <= 128; ++zc)
+        if (cost(zc) < least) least = cost(zc), best = zc;
+    return best;
+}
+
+// FP32 chunk.  Below 192^3 the pass runs out of L2 and its time is latency and
+// the last CTA's sum over all others: the shortest chunk whose CTAs are all on
+// the GPU at once, one per SM while that is at most six field-planes, else two
+// per SM (us, two fields: 48^3 11.0 -> 9.7 with 1 plane, not 3, 64^3 12.0 -> 10.0 with
+// 2, not 4, 128^3 25.7 -> 20.3 with 7, not 4, 160^3 61 -> 44 with 16, not 4).
+// Larger lattices: at least four planes (the planes on either side of a chunk are
+// traffic) and several waves of CTAs.
+static int f32_chunk(int N, int nf, int tiles, int sms)
+{
+    if (N < 192) {
+        auto shortest = [&](long ctas) {
+            int zc = 1;
+            while (zc < N && (long)tiles * ((N + zc - 1) / zc) > ctas) ++zc;
+            return zc;
+        };
+        const int zc = shortest(sms);
+        return zc * nf <= 6 ? zc : shortest(2L * sms);
+    }
+    int zc = 128;
+    while (zc > 4 && (long)tiles * ((N + zc - 1) / zc) < 8L * sms) zc /= 2;
+    return zc;
 }
 
 PassGeom pass_geometry(int N, int elem_bytes, int sm_count, int nf, const PassTuning &t)
@@ -61,24 +108,31 @@ PassGeom pass_geometry(int N, int elem_bytes, int sm_count, int nf, const PassTu
     g.threads = (t.variant == kVariantLdg && t.threads == 512) ? 512 : 256;
     const int threads = t.variant == kVariantTma ? 32 * g.cwarps : g.threads;
     const int txt_max = (t.variant == kVariantLdg && (t.txt == 8 || t.txt == 16)) ? t.txt : 32;
-    g.txt = per_row < txt_max ? per_row : txt_max;
+    g.tile_x = g.txt = per_row < txt_max ? per_row : txt_max;
+    if (t.variant == kVariantLdg && txt_max == 32) g.txt = even_row_tile(per_row);
     g.ty = threads / g.txt;
     if (g.ty > N) g.ty = N;
     const int gx = (per_row + g.txt - 1) / g.txt;
-    const int gy = (N + g.ty - 1) / g.ty;
-    // z-chunk: long enough to amortise the two extra planes, short enough
-    // for several waves of CTAs over the GPU.  FP64 passes are bound by the
-    // FP64 pipe, so a small lattice spreads down to one plane per CTA to reach
-    // more SMs (the extra halo planes cost loads, not FP64 work); FP32 passes
-    // keep at least 4 planes, since for them the halo planes are traffic.
-    int zc = t.zc > 0 ? t.zc : (N < 128 ? N : 128);
-    if (t.zc <= 0) {
-        const long target = 8L * (sm_count > 0 ? sm_count : 152);
-        const int zmin = elem_bytes == 8 ? 1 : 4;
-        while (zc > zmin && (long)gx * gy * ((N + zc - 1) / zc) < target) zc /= 2;
+    int gy = (N + g.ty - 1) / g.ty;
+    const int sms = sm_count > 0 ? sm_count : 152;
+    const bool f64_stream = t.variant == kVariantLdg && elem_bytes == 8;
+    int zc = t.zc;
+    if (zc <= 0) {
+        if (f64_stream) {
+            zc = f64_chunk(N, gx, g.txt, g.ty, sms);
+        } else if (t.variant == kVariantLdg) {
+            zc = f32_chunk(N, nf, gx * gy, sms);
+        } else {  // TMA: long enough to amortise the two extra planes, short enough for several waves
+            zc = N < 128 ? N : 128;
+            while (zc > 4 && (long)gx * gy * ((N + zc - 1) / zc) < 8L * sms) zc /= 2;
+        }
     }
     if (zc > N) zc = N;
     g.zc = zc;
+    if (f64_stream) {
+        g.ty = f64_tile_rows(N, gx, g.txt, g.ty, zc, sms);
+        gy = (N + g.ty - 1) / g.ty;
+    }
     g.grid = dim3(gx, gy, (N + zc - 1) / zc);
     g.nblocks = g.grid.x * g.grid.y * g.grid.z;
     g.stages = 0;

@@ -22,8 +22,10 @@
 #include <math.h>
 
 #include <atomic>
+#include <utility>
 
 #include "tl_internal.cuh"
+#include "tl_scale.cuh"
 
 namespace tl {
 
@@ -80,85 +82,136 @@ __device__ __forceinline__ void store_vec_cs(double *p, const double (&v)[2])
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-__device__ __forceinline__ double warp_sum(double v)
+// Warp sums of NQ values at once, in lane i < NQ the sum of v[i]: each exchange
+// also halves the values a lane carries on, so that NQ <= 4 (8) of them take 6
+// (9) additions instead of 5 NQ.  GB300's FP64 pipe takes two lanes a clock, so an
+// FP64 addition of a warp holds it for 16 clocks whatever its lanes do.
+template <int NQ, typename A>
+__device__ __forceinline__ A warp_sums(const A (&v)[NQ])
 {
+    constexpr int M = NQ <= 4 ? 4 : 8;
+    static_assert(NQ <= 8, "at most eight sums at once");
+    const int lane = threadIdx.x & 31;
+    A w[M];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// x^e: integer exponents up to 16 in magnitude by repeated squaring (a few
-// multiplications instead of a pow() on the FP64 unit, which this last-CTA
-// tail would otherwise serialise every pass); other exponents by pow().
-__device__ __forceinline__ double powe(double x, double e)
-{
-    const double r = rint(e);
-    if (r == e && fabs(r) <= 16.0) {
-        int n = (int)fabs(r);
-        double acc = 1.0, b = x;
-        while (n) {
-            if (n & 1) acc *= b;
-            b *= b;
-            n >>= 1;
+    for (int i = 0; i < M; ++i) w[i] = i < NQ ? v[i < NQ ? i : 0] : (A)0;
+    int o = 16;
+#pragma unroll
+    for (int h = M / 2; h > 0; h /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const A keep = up ? w[i + h] : w[i], send = up ? w[i] : w[i + h];
+            w[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
-        return r < 0.0 ? 1.0 / acc : acc;
     }
-    return pow(x, e);
+#pragma unroll
+    for (; o > 0; o /= 2) w[0] += __shfl_xor_sync(0xffffffffu, w[0], o);
+    return __shfl_sync(0xffffffffu, w[0], (lane * (32 / M)) & 31);  // from the first lane that holds sum `lane`
 }
 
-// Scale-factor update and next-pass coefficients (one thread of the last CTA).
-// tot: raw lattice sums  [sum pi_int_f^2, sum |grad+ phi_f|^2 dx^2, sum V].
-static __device__ void finalize(const Model &m, const PassCoef &c, Scalars *sc, const double *tot)
+// Programmatic dependent launch: a pass may start while the one before it runs
+// out (its CTAs take the SMs as they fall free) and waits here until that one is
+// complete and its writes are visible; then its own successor may start.
+__device__ __forceinline__ void pass_begin()
 {
-    const int nf = m.nf;
-    const double n3 = (double)m.N * (double)m.N * (double)m.N;
-    const double a = sc->a;
-    double E[kMaxQ];
-    double K = 0.0, G = 0.0;
-    bool finite = true;
-    for (int f = 0; f < nf; ++f) {
-        E[f] = 0.5 * sc->wk * (tot[f] / n3);
-        E[nf + f] = 0.5 * sc->wg * m.inv_dx2 * (tot[nf + f] / n3);
-        K += E[f];
-        G += E[nf + f];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// The scalars the end of a pass starts from.
+struct PassEnd {
+    double a, b, wk, wg, pf, ph, ia, time, pending_dt;
+    int status;
+};
+
+// Energies, scale-factor update and next-pass coefficients, by one warp of the
+// last CTA; lane i < NQ brings the lattice sum of quantity i: [sum pi_int_f^2,
+// sum |grad+ phi_f|^2 dx^2, sum V].
+//
+// Every pass ends in this serial tail, and an FP64 operation waits 65 clocks for
+// the one before it (a division 550), so that the tail is a good part of a
+// small lattice's pass: the energies are formed in one lane each, the powers
+// of the new scale factor too, and nothing is divided.
+template <int NQ>
+static __device__ __forceinline__ void finalize(const Model &m, const PassCoef &c, Scalars *sc, const PassEnd &was,
+                                                double tot)
+{
+    constexpr int NF = (NQ - 1) / 2;
+    const int lane = threadIdx.x & 31;
+    const double weight = lane < NF ? 0.5 * was.wk : lane < 2 * NF ? 0.5 * was.wg * m.inv_dx2 : 1.0;
+    const double E = weight * m.inv_n3 * tot;
+    const bool finite = __all_sync(0xffffffffu, lane >= NQ || isfinite(E));
+    if (c.integer_time && lane < NQ) sc->E[lane] = E;
+    double K = __shfl_sync(0xffffffffu, E, 0), G = __shfl_sync(0xffffffffu, E, NF);
+    if constexpr (NF > 1) {
+#pragma unroll
+        for (int f = 1; f < NF; ++f) {
+            K += __shfl_sync(0xffffffffu, E, f);
+            G += __shfl_sync(0xffffffffu, E, NF + f);
+        }
     }
-    const double V = tot[2 * nf] / n3;
-    E[2 * nf] = V;
-    for (int i = 0; i < 2 * nf + 1; ++i) {
-        finite = finite && isfinite(E[i]);
-        if (c.integer_time) sc->E[i] = E[i];
-    }
-    if (!finite && sc->status == TL_OK) sc->status = TL_EUNSTABLE;
-    sc->time += sc->pending_dt;
+    const double V = __shfl_sync(0xffffffffu, E, 2 * NF);
+    double drift = c.dnext_dt, hubble = 0.0;
     if (m.expanding) {
-        const double al = m.alpha;
+        const double al = m.alpha, a = was.a;
         const double rho = K + G + V;
-        double b = sc->b, b_eval;
+        double b, b_eval;
         if (c.set_b_from_constraint) {
-            b = powe(a, 1.0 + al) * sqrt(m.mu2 * rho / 3.0);
-            b_eval = b;
+            b = b_eval = sqrt(was.ph * a * a * (m.mu2 * rho / 3.0));
         } else {
-            const double fb = powe(a, 2.0 * al + 1.0) * (m.mu2 / 3.0) * ((al - 2.0) * K + al * G + (al + 1.0) * V);
-            b_eval = b + c.hb_dt * fb;
-            b = b + c.edt * fb;
+            const double f = was.pf * m.mu2_3;
+            const double fb = fma(al + 1.0, V, fma(al, G, (al - 2.0) * K));
+            b_eval = fma(c.hb_dt * f, fb, was.b);
+            b = fma(c.edt * f, fb, was.b);
         }
-        if (c.integer_time) {
-            const double H2 = (b_eval / a) * (b_eval / a);
-            sc->hubble = fabs(H2 - powe(a, 2.0 * al) * m.mu2 * rho / 3.0) / H2;
+        const double an = fma(c.dnext_dt, b, a);
+        const double H = b_eval * was.ia, H2 = H * H;
+        const double r = write_scale_powers(m, sc, an, 0.5 * (a + an), H2);
+        drift *= __shfl_sync(0xffffffffu, r, kScalePowers);
+        hubble = fabs(H2 - was.ph * m.mu2_3 * rho) * __shfl_sync(0xffffffffu, r, kScalePowers + 1);
+        if (lane == 0) {
+            sc->a = an;
+            sc->b = b;
         }
-        const double an = a + c.dnext_dt * b;
-        sc->drift = c.dnext_dt * powe(0.5 * (a + an), al - 3.0);
-        sc->a = an;
-        sc->b = b;
-        sc->wl = powe(an, 1.0 + al);
-        sc->wv = powe(an, 3.0 + al);
-        sc->wk = powe(an, -6.0);
-        sc->wg = powe(an, -2.0);
-    } else {
-        sc->drift = c.dnext_dt;
-        sc->hubble = 0.0;
     }
-    sc->pending_dt = c.dnext_dt;
+    if (lane == 0) {
+        if (!finite && was.status == TL_OK) sc->status = TL_EUNSTABLE;
+        sc->time = was.time + was.pending_dt;
+        sc->pending_dt = c.dnext_dt;
+        sc->drift = drift;
+        if (c.integer_time || !m.expanding) sc->hubble = hubble;
+        sc->ticket = 0u;
+    }
+}
+
+// The end of a tile, by one warp: lane i < NQ brings the tile's sum of quantity
+// i.  It goes into the tile's slot (slots[i][tile]); the lattice's last tile to
+// arrive sums all slots in a fixed order (lanes in strides of 32, then the warp
+// tree) and runs finalize().  Deterministic for a given launch geometry.
+template <int NQ>
+__device__ __forceinline__ void finish_tile(double sum, const Model &m, const PassCoef &c, Scalars *sc, double *slots,
+                                            unsigned bid, unsigned nblocks)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane < NQ) __stcg(slots + (size_t)lane * nblocks + bid, sum);
+    __syncwarp();
+    unsigned ticket = 0;
+    if (lane == 0) {
+        __threadfence();
+        ticket = atomicAdd(&sc->ticket, 1u);
+    }
+    if (__shfl_sync(0xffffffffu, ticket, 0) != nblocks - 1) return;
+    __threadfence();
+    const PassEnd was{sc->a, sc->b, sc->wk, sc->wg, sc->pf, sc->ph, sc->ia, sc->time, sc->pending_dt, sc->status};
+    double part[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) part[i] = 0.0;
+#pragma unroll 4
+    for (unsigned b = lane; b < nblocks; b += 32)
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) part[i] += __ldcg(slots + (size_t)i * nblocks + b);
+    finalize<NQ>(m, c, sc, was, warp_sums<NQ>(part));
 }
 
 // ---- pieces shared by both pass variants ------------------------------------
@@ -174,32 +227,77 @@ struct Coefs {
     T wm2[NF];   // a^(3+alpha) m2
 };
 
-template <typename T, int NF>
-__device__ __forceinline__ Coefs<T, NF> make_coefs(const Model &m, const PassCoef &c, const Scalars *sc)
+// Formed once per CTA by one warp, a coefficient per lane, and read by every
+// thread from shared memory: the products and conversions run on the FP64 pipe,
+// where a warp instruction takes 16 clocks (20 of them in each of 8 warps were
+// 1.3 us at the start of every CTA, and with three fields the compiler repeated
+// eight conversions per plane to save registers: 39% of the FP64 pipe).
+constexpr int kCoefs = 20;
+
+template <typename T>
+__device__ __forceinline__ void share_coefs(T *shared, const Model &m, const PassCoef &c, const Scalars *sc)
 {
-    Coefs<T, NF> k;
-    k.drift = (T)sc->drift;
-    k.wlx = (T)(sc->wl * m.inv_dx2);
-    k.wv = (T)sc->wv;
-    k.kdt = (T)c.kdt;
-    k.hdt = (T)c.hdt;
-    k.lam = (T)m.lambda;
-    k.q = (T)m.q;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        k.m2[f] = (T)m.m2[f];
-        k.hm2[f] = (T)(0.5 * m.m2[f]);
-    }
-    k.qlam = (T)(0.25 * m.lambda);
-    k.hq = (T)(0.5 * m.q);
-    k.wlam = (T)(sc->wv * m.lambda);
-    k.wq = (T)(sc->wv * m.q);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) k.wm2[f] = (T)(sc->wv * m.m2[f]);
-    return k;
+    const int lane = threadIdx.x & 31;
+    if (lane >= kCoefs) return;
+    const double s = lane == 0 ? sc->drift : lane == 1 ? sc->wl : lane == 2 || lane >= 15 ? sc->wv : 1.0;
+    double f = 1.0;
+    if (lane == 1) f = m.inv_dx2;
+    else if (lane == 3) f = c.kdt;
+    else if (lane == 4) f = c.hdt;
+    else if (lane == 5 || lane == 15) f = m.lambda;
+    else if (lane == 6 || lane == 16) f = m.q;
+    else if (lane == 10) f = 0.25 * m.lambda;
+    else if (lane == 11) f = 0.5 * m.q;
+    else if (lane == 7 || lane == 17) f = m.m2[0];
+    else if (lane == 8 || lane == 18) f = m.m2[1];
+    else if (lane == 9 || lane == 19) f = m.m2[2];
+    else if (lane == 12) f = 0.5 * m.m2[0];
+    else if (lane == 13) f = 0.5 * m.m2[1];
+    else if (lane == 14) f = 0.5 * m.m2[2];
+    shared[lane] = (T)(s * f);
 }
 
-
+template <typename T, int NF, bool PIN = (NF <= 2)>
+__device__ __forceinline__ Coefs<T, NF> load_coefs(const T *shared)
+{
+    Coefs<T, NF> k;
+    k.drift = shared[0];
+    k.wlx = shared[1];
+    k.wv = shared[2];
+    k.kdt = shared[3];
+    k.hdt = shared[4];
+    k.lam = shared[5];
+    k.q = shared[6];
+    k.qlam = shared[10];
+    k.hq = shared[11];
+    k.wlam = shared[15];
+    k.wq = shared[16];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        k.m2[f] = shared[7 + f];
+        k.hm2[f] = shared[12 + f];
+        k.wm2[f] = shared[17 + f];
+    }
+    if (PIN) {
+        auto pin = [](T &x) {
+            if constexpr (sizeof(T) == 4) asm volatile("" : "+f"(x));
+            else asm volatile("" : "+d"(x));
+        };
+        pin(k.drift), pin(k.wlx), pin(k.kdt), pin(k.hdt);
+        if constexpr (sizeof(T) == 4) {
+            pin(k.wv), pin(k.lam);
+            if (NF > 1) pin(k.q);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) pin(k.m2[f]);
+        } else {
+            pin(k.qlam), pin(k.wlam);
+            if (NF > 1) pin(k.hq), pin(k.wq);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) pin(k.hm2[f]), pin(k.wm2[f]);
+        }
+    }
+    return k;
+}
 
 // Update W consecutive sites of one row of plane z, all fields: Laplacian from
 // the six neighbours (differences first, so FP32 keeps the small gradients
@@ -303,72 +401,47 @@ __device__ __forceinline__ void site_update(const Coefs<T, NF> &k, const T (&cu)
     }
 }
 
-// CTA sum in a fixed order (warp trees, then warps in index order) into this
-// CTA's slot; the last CTA to arrive sums all slots in index order and runs
-// finalize().  Deterministic for a given launch geometry.
-// F32TREE (FP32 lattices): the warp tree runs in FP32 and each warp adds its
-// sum to the CTA's FP64 total -- thread sums (FP32 in-thread, promoted to FP64
-// every 16 planes), FP32 warp tree, FP64 from there on; FP64 lattices keep the
-// whole tree in FP64.
-template <int NQ, bool F32TREE = false>
-__device__ __forceinline__ void cta_reduce_finalize(const double (&accd)[NQ], const Model &m, const PassCoef &c,
-                                                    Scalars *sc, double *slots, unsigned bid, unsigned nblocks)
+// Sums of a tile over the first nwarps warps of its CTA, in a fixed order (warp
+// trees, then warps in index order), and the end of the tile (finish_tile) by
+// warp 0.  FP32 lattices: acc holds a thread's sums if the tile has at most
+// kFlush planes, accd otherwise (sums of kFlush planes in FP32, then FP64); the
+// warp tree runs in FP32 and each warp adds its sum to the tile's FP64 total.
+// FP64 lattices keep the whole tree in FP64.  sync: a barrier of those warps.
+constexpr int kFlush = 16;
+
+template <int NQ, typename T, typename Sync>
+__device__ __forceinline__ double tile_sum(const T (&acc)[NQ], const double (&accd)[NQ], bool flushed, int nwarps,
+                                           double (*red)[NQ], Sync sync)  // in lane i < NQ of warp 0
 {
-    __shared__ double red[32][NQ];
-    __shared__ bool last;
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int nwarps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T v[NQ];
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-        double v;
-        if constexpr (F32TREE) {
-            float w = (float)accd[i];
+    for (int i = 0; i < NQ; ++i) v[i] = acc[i];
+    if (flushed) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            v = (double)w;
-        } else {
-            v = warp_sum(accd[i]);
-        }
-        if (lane == 0) red[warp][i] = v;
+        for (int i = 0; i < NQ; ++i) v[i] = (T)accd[i];
     }
-    __syncthreads();
-    if (tid < NQ) {
-        double s = 0.0;
-        for (int w = 0; w < nwarps; ++w) s += red[w][tid];
-        slots[(size_t)bid * NQ + tid] = s;
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = (atomicAdd(&sc->ticket, 1u) == nblocks - 1);
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        double part[NQ];
+    const T w = warp_sums<NQ>(v);
+    if (lane < NQ) red[warp][lane] = (double)w;
+    sync();
+    if (warp != 0 || lane >= NQ) return 0.0;
+    double s[4];  // four chains: additions wait for each other
 #pragma unroll
-        for (int i = 0; i < NQ; ++i) part[i] = 0.0;
-        for (unsigned b = tid; b < nblocks; b += blockDim.x)
+    for (int k = 0; k < 4; ++k) s[k] = k < nwarps ? red[k][lane] : 0.0;
+    for (int k = 4; k < nwarps; k += 4)
 #pragma unroll
-            for (int i = 0; i < NQ; ++i) part[i] += __ldcg(slots + (size_t)b * NQ + i);
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) {
-            double v = warp_sum(part[i]);
-            if (lane == 0) red[warp][i] = v;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double tot[kMaxQ];
-            for (int i = 0; i < NQ; ++i) {
-                double s = 0.0;
-                for (int w = 0; w < nwarps; ++w) s += red[w][i];
-                tot[i] = s;
-            }
-            finalize(m, c, sc, tot);
-            sc->ticket = 0u;
-            __threadfence();
-        }
-    }
-    __syncthreads();  // red[] and last may be reused by the next tile of a persistent CTA
+        for (int i = 0; i < 4; ++i)
+            if (k + i < nwarps) s[i] += red[k + i][lane];
+    return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+template <int NQ, typename T, typename Sync>
+__device__ __forceinline__ void reduce_tile(const T (&acc)[NQ], const double (&accd)[NQ], bool flushed, int nwarps,
+                                            double (*red)[NQ], Sync sync, const Model &m, const PassCoef &c, Scalars *sc,
+                                            double *slots, unsigned bid, unsigned nblocks)
+{
+    const double s = tile_sum<NQ>(acc, accd, flushed, nwarps, red, sync);
+    if (threadIdx.x < 32) finish_tile<NQ>(s, m, c, sc, slots, bid, nblocks);
 }
 
 __device__ __forceinline__ unsigned grid_bid() { return blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z); }
@@ -433,26 +506,55 @@ __device__ __forceinline__ void ldg_tile(const Model &m, const FieldPtrs &fp, co
         return reinterpret_cast<T *>(ring_raw) + ((size_t)((d * NF + f) * 2 + a) * blockDim.x + tid) * W;
     };
 
+    __shared__ T coefs[kCoefs];
+    __shared__ double red[512 / 32][NQ];
+    const bool flushed = z1 - z0 > kFlush;
     double accd[NQ];
+    T acc[NQ];
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) accd[i] = 0.0;
+    for (int i = 0; i < NQ; ++i) {
+        accd[i] = 0.0;
+        acc[i] = (T)0;
+    }
+    const T *phs[NF], *pis[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        phs[f] = static_cast<const T *>(fp.phi_in[f]);
+        pis[f] = static_cast<const T *>(fp.pi_in[f]);
+    }
+    const size_t NN = (size_t)m.pplane;
+    const size_t P = (size_t)m.pitch;
+    const size_t row = (size_t)y * P;
+    // the stored words of the first two planes, on their way while the coefficients are formed
+    T zm[NF][W], cu[NF][W], zp[NF][W], pc[NF][W], pm[NF][W];
+    if (active) {
+        const size_t below = (size_t)((z0 == 0) ? N - 1 : z0 - 1) * NN + row + x0, first = (size_t)z0 * NN + row + x0;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            load_vec(phs[f] + below, zm[f]);
+            load_vec(pis[f] + below, pm[f]);
+            load_vec(phs[f] + first, cu[f]);
+            load_vec(pis[f] + first, pc[f]);
+        }
+    }
+    if (tid < 32) share_coefs(coefs, m, c, sc);
+    __syncthreads();
 
     if (active) {
-        const Coefs<T, NF> k = make_coefs<T, NF>(m, c, sc);
-        const T *phs[NF], *pis[NF];
+        const Coefs<T, NF> k = load_coefs<T, NF>(coefs);
         T *pho[NF], *pio[NF];
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            phs[f] = static_cast<const T *>(fp.phi_in[f]);
-            pis[f] = static_cast<const T *>(fp.pi_in[f]);
             pho[f] = static_cast<T *>(fp.phi_out[f]);
             pio[f] = static_cast<T *>(fp.pi_out[f]);
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                zm[f][j] = fma_t(k.drift, pm[f][j], zm[f][j]);
+                cu[f][j] = fma_t(k.drift, pc[f][j], cu[f][j]);
+            }
         }
-        const size_t NN = (size_t)m.pplane;
-        const size_t P = (size_t)m.pitch;
         const int xl = (x0 == 0) ? N - 1 : x0 - 1;
         const int xr = (x0 + W == N) ? 0 : x0 + W;
-        const size_t row = (size_t)y * P;
         const size_t rowm = (size_t)((y == 0) ? N - 1 : y - 1) * P;
         const size_t rowp = (size_t)((y + 1 == N) ? 0 : y + 1) * P;
         auto cur_vec = [&](int f, size_t off, T (&o)[W]) {
@@ -479,28 +581,10 @@ __device__ __forceinline__ void ldg_tile(const Model &m, const FieldPtrs &fp, co
             cp_async_commit();
         };
 
-        T zm[NF][W], cu[NF][W], zp[NF][W], pc[NF][W];
-        {
-            const size_t pm = (size_t)((z0 == 0) ? N - 1 : z0 - 1) * NN;
-            const size_t p0 = (size_t)z0 * NN;
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                cur_vec(f, pm + row + x0, zm[f]);
-                T a[W];
-                load_vec(phs[f] + p0 + row + x0, a);
-                load_vec(pis[f] + p0 + row + x0, pc[f]);
-#pragma unroll
-                for (int j = 0; j < W; ++j) cu[f][j] = fma_t(k.drift, pc[f][j], a[j]);
-            }
-        }
         if (D > 0) {
 #pragma unroll
             for (int d = 0; d < D; ++d) prefetch(z0 + 1 + d, d);
         }
-        T acc[NQ];
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) acc[i] = (T)0;
-
         int d = 0;  // ring slot holding plane z+1
         for (int z = z0; z < z1; ++z) {
             const size_t pz = (size_t)z * NN;
@@ -546,7 +630,7 @@ __device__ __forceinline__ void ldg_tile(const Model &m, const FieldPtrs &fp, co
                 }
                 if (m.ghosts) store_ghosts<T, NF, W>(pho, pio, cu, pnew, pz, x0, y, N, (long long)P);
             }
-            if (((z - z0) & 15) == 15) {
+            if (flushed && ((z - z0) & (kFlush - 1)) == kFlush - 1) {
 #pragma unroll
                 for (int i = 0; i < NQ; ++i) {
                     accd[i] += (double)acc[i];
@@ -563,10 +647,12 @@ __device__ __forceinline__ void ldg_tile(const Model &m, const FieldPtrs &fp, co
                 }
         }
         if (D > 0) cp_async_wait<0>();
+        if (flushed) {
 #pragma unroll
-        for (int i = 0; i < NQ; ++i) accd[i] += (double)acc[i];
+            for (int i = 0; i < NQ; ++i) accd[i] += (double)acc[i];
+        }
     }
-    cta_reduce_finalize<NQ, sizeof(T) == 4>(accd, m, c, sc, slots, bid, nblocks);
+    reduce_tile<NQ>(acc, accd, flushed, (int)blockDim.x >> 5, red, [] { __syncthreads(); }, m, c, sc, slots, bid, nblocks);
 }
 
 template <typename T, int NF, bool MEASURE, int D, int NT>
@@ -574,6 +660,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) fused_pass_ldg(Model m, FieldPtr
                                                             Scalars *sc, double *slots)
 {
     extern __shared__ __align__(16) unsigned char ring_raw[];
+    pass_begin();
     ldg_tile<T, NF, MEASURE, D>(m, fp, c, txt, ty, zc, blockIdx.x, blockIdx.y, blockIdx.z, grid_bid(), grid_nblocks(),
                                 sc, slots, ring_raw);
 }
@@ -614,6 +701,7 @@ __global__ void __launch_bounds__(256, 2) fused_pass_group(const BatchJob *__res
         __syncthreads();
     }
     const unsigned *first = staged ? s_first : first_item;
+    pass_begin();
     for (unsigned item = blockIdx.x; item < total; item += gridDim.x) {
         int lo = 0, hi = njobs - 1;  // last job whose first item <= item
         while (lo < hi) {
@@ -627,7 +715,25 @@ __global__ void __launch_bounds__(256, 2) fused_pass_group(const BatchJob *__res
         const int by = (int)((local / (unsigned)j.gx) % (unsigned)j.gy);
         const int bz = (int)(local / ((unsigned)j.gx * (unsigned)j.gy));
         ldg_tile<T, NF, false, D>(j.m, j.fp, c, j.txt, j.ty, j.zc, bx, by, bz, local, j.nblocks, j.sc, j.slots, ring);
+        __syncthreads();  // the shared sums and coefficients are the next item's
     }
+}
+
+// Launch with programmatic dependent launch allowed (see pass_begin).
+template <typename... P, typename... A>
+static cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
 }
 
 // Enqueue one grouped pass (see launch_group).
@@ -654,8 +760,7 @@ static cudaError_t launch_group_t(int prefetch, const BatchJob *jobs, const unsi
             }
         }
     }
-    kern<<<grid, 256, smem, s>>>(jobs, first_item, njobs, total, c);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3((unsigned)grid), 256, smem, s, jobs, first_item, njobs, total, c);
 }
 
 // ---- PTX helpers for asynchronous copies ---------------------------------------
@@ -736,70 +841,9 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
 
 constexpr int kMaxStages = 8;
 
-// The fixed-order sum of cta_reduce_finalize for the compute warps of a TMA
-// CTA alone (threads 0 .. nthr-1, named barrier 1), so that the producer warp
-// can go on loading the next tile's planes meanwhile.  The same numbers as the
-// whole-CTA form: the producer warp's share was zero.  The last tile to arrive
-// sums all slots with a fixed stride of 128 threads.
-template <int NQ, bool F32TREE>
-__device__ __forceinline__ void consumer_reduce_finalize(const double (&accd)[NQ], const Model &m, const PassCoef &c,
-                                                         Scalars *sc, double *slots, unsigned bid, unsigned nblocks,
-                                                         unsigned nthr)
-{
-    __shared__ double red[32][NQ];
-    __shared__ bool last;
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int nwarps = (int)(nthr >> 5);
-    auto sync = [&] { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); };
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-        double v;
-        if constexpr (F32TREE) {
-            float w = (float)accd[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            v = (double)w;
-        } else {
-            v = warp_sum(accd[i]);
-        }
-        if (lane == 0) red[warp][i] = v;
-    }
-    sync();
-    if (tid < NQ) {
-        double s = 0.0;
-        for (int w = 0; w < nwarps; ++w) s += red[w][tid];
-        slots[(size_t)bid * NQ + tid] = s;
-    }
-    __threadfence();
-    sync();
-    if (tid == 0) last = (atomicAdd(&sc->ticket, 1u) == nblocks - 1);
-    sync();
-    if (last) {
-        __threadfence();
-        double part[NQ];
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) part[i] = 0.0;
-        if (tid < 128)
-            for (unsigned b = tid; b < nblocks; b += 128)
-#pragma unroll
-                for (int i = 0; i < NQ; ++i) part[i] += __ldcg(slots + (size_t)b * NQ + i);
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) {
-            double v = warp_sum(part[i]);
-            if (lane == 0 && warp < 4) red[warp][i] = v;
-        }
-        sync();
-        if (tid == 0) {
-            double tot[kMaxQ];
-            for (int i = 0; i < NQ; ++i) tot[i] = ((red[0][i] + red[1][i]) + red[2][i]) + red[3][i];
-            finalize(m, c, sc, tot);
-            sc->ticket = 0u;
-            __threadfence();
-        }
-    }
-    sync();  // red[] and last are reused by the next tile
-}
+// A barrier of the compute warps of a TMA CTA alone (threads 0 .. nthr-1): the
+// producer warp goes on, or has left.
+__device__ __forceinline__ void consumer_sync(unsigned nthr) { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); }
 
 // One CTA tile (bx, by, bz) of the TMA pass; bid/nblocks index the tile among
 // the lattice's tiles for the reduction; maps points to the tensor maps of the
@@ -862,9 +906,21 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
     }
     __syncthreads();
 
+    pass_begin();
+    __shared__ T coefs[kCoefs];
+    __shared__ double red[16][NQ];
+    if (!producer) {
+        if (tid < 32) share_coefs(coefs, m, c, sc);
+        consumer_sync((unsigned)CW * 32u);
+    }
+    constexpr bool flushed = true;
     double accd[NQ];
+    T acc[NQ];
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) accd[i] = 0.0;
+    for (int i = 0; i < NQ; ++i) {
+        accd[i] = 0.0;
+        acc[i] = (T)0;
+    }
     int issued = 0;
 
     if (producer) {
@@ -929,7 +985,7 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
         const bool col_r = edge && (tx == txt - 1 || x0 + W >= N);
         const int col = (tyi + 1) * W;  // this thread's row in a halo column
         const int src_l = own_l ? lane : lane - 1, src_r = own_r ? lane : lane + 1;
-        const Coefs<T, NF> k = make_coefs<T, NF>(m, c, sc);
+        const Coefs<T, NF> k = load_coefs<T, NF>(coefs);
         const int ctr = (tyi + 1) * rowe + (edge ? 0 : W) + tx * W;
         const size_t P = (size_t)m.pitch, PP = (size_t)m.pplane;
         T *pho[NF], *pio[NF];
@@ -939,9 +995,6 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
             pio[f] = static_cast<T *>(fp.pi_out[f]);
         }
         T zm[NF][W], cu[NF][W], zp[NF][W], pc[NF][W], pn[NF][W];
-        T acc[NQ];
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) acc[i] = (T)0;
         auto centre = [&](int s, T (&ph)[NF][W], T (&pp)[NF][W]) {
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
@@ -979,10 +1032,10 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
         adv_w();
         if (!ok) s_failed = 1;
         release(0);
-        // blocks of 16 planes: after each, the FP32 energy sums go into FP64
+        // blocks of kFlush planes: after each, the FP32 energy sums go into FP64
         bool stop = false;
-        for (int zb = z0; zb < z1 && !stop; zb += 16) {
-        const int ze = min(zb + 16, z1);
+        for (int zb = z0; zb < z1 && !stop; zb += kFlush) {
+        const int ze = min(zb + kFlush, z1);
         for (int z = zb; z < ze; ++z) {
             if (__any_sync(0xffffffffu, s_failed != 0)) {  // warp-uniform exit
                 stop = true;
@@ -1042,8 +1095,6 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
             acc[i] = (T)0;
         }
         }
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) accd[i] += (double)acc[i];
     }
     if (producer) {
         // After a timeout, wait (bounded) for the copies still in flight before the
@@ -1053,7 +1104,7 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
                 mbar_wait_bounded(&full[kk % S], (kk / S) & 1u, sc);
         return;
     }
-    consumer_reduce_finalize<NQ, sizeof(T) == 4>(accd, m, c, sc, slots, bid, nblocks, (unsigned)CW * 32u);
+    reduce_tile<NQ>(acc, accd, flushed, CW, red, [&] { consumer_sync((unsigned)CW * 32u); }, m, c, sc, slots, bid, nblocks);
 }
 
 // Tiles first, first + stride, ... (< nitems) of the TMA pass, in a CTA whose
@@ -1106,6 +1157,7 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
     }
     __syncthreads();
 
+    pass_begin();
     if (producer) {
         if (lane == 0) {
             if constexpr (GLOBAL_MAPS) {
@@ -1181,6 +1233,10 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
     }
 
     const unsigned nthr = (unsigned)CW * 32u;
+    __shared__ T coefs[kCoefs];
+    __shared__ double red[16][NQ];
+    if (tid < 32) share_coefs(coefs, m, c, sc);
+    consumer_sync(nthr);
     const size_t P = (size_t)m.pitch, PP = (size_t)m.pplane;
     T *pho[NF], *pio[NF];
 #pragma unroll
@@ -1217,9 +1273,14 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
         const int y = y_tile + tyi;
         const bool active = (tyi < ty) && (x0 < N) && (y < N);
         const bool warp_active = __any_sync(0xffffffffu, active);
+        constexpr bool flushed = true;
         double accd[NQ];
+        T acc[NQ];
 #pragma unroll
-        for (int i = 0; i < NQ; ++i) accd[i] = 0.0;
+        for (int i = 0; i < NQ; ++i) {
+            accd[i] = 0.0;
+            acc[i] = (T)0;
+        }
         if (warp_active) {
             // x-neighbours: the left site is the last one of the thread to the
             // left in the same row and warp, the right site the first one of the
@@ -1233,12 +1294,9 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
             const bool col_r = edge && (tx == txt - 1 || x0 + W >= N);
             const int col = (tyi + 1) * W;  // this thread's row in a halo column
             const int src_l = own_l ? lane : lane - 1, src_r = own_r ? lane : lane + 1;
-            const Coefs<T, NF> k = make_coefs<T, NF>(m, c, sc);
+            const Coefs<T, NF> k = load_coefs<T, NF>(coefs);
             const int ctr = (tyi + 1) * rowe + (edge ? 0 : W) + tx * W;
             T zm[NF][W], cu[NF][W], zp[NF][W], pc[NF][W], pn[NF][W];
-            T acc[NQ];
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) acc[i] = (T)0;
             auto centre = [&](int s, T (&ph)[NF][W], T (&pp)[NF][W]) {
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
@@ -1301,7 +1359,7 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
                         }
                         if (m.ghosts) store_ghosts<T, NF, W>(pho, pio, cu, pnew, pz, x0, y, N, (long long)P);
                     }
-                    if (((z - z0) & 15) == 15) {
+                    if (((z - z0) & (kFlush - 1)) == kFlush - 1) {
 #pragma unroll
                         for (int i = 0; i < NQ; ++i) {
                             accd[i] += (double)acc[i];
@@ -1333,9 +1391,9 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
                 release_next();
             }
         }
-        consumer_reduce_finalize<NQ, sizeof(T) == 4>(accd, m, c, sc, slots, item, nitems, nthr);
+        reduce_tile<NQ>(acc, accd, flushed, CW, red, [&] { consumer_sync(nthr); }, m, c, sc, slots, item, nitems);
         if (tid == 0) s_stop = s_failed;
-        asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+        consumer_sync(nthr);
         if (s_stop) break;
     }
 }
@@ -1444,9 +1502,8 @@ static cudaError_t launch_tma(const Model &m, const FieldPtrs &fp, const PassCoe
     // frees up, which keeps the CTAs in flight a compact band of neighbouring
     // tiles (their halo rows meet in L2).  A persistent grid walking tiles b,
     // b + grid, ... measured 11-25% slower: its CTAs drift apart.
-    kern<<<g.nblocks, threads, g.smem, s>>>(m, fp, c, g.txt, g.ty, g.zc, g.stages, g.lpad, maps, sc, slots,
-                                            (int)g.grid.x, (int)g.grid.y, g.nblocks);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(g.nblocks), threads, g.smem, s, m, fp, c, g.txt, g.ty, g.zc, g.stages, g.lpad, maps,
+                            sc, slots, (int)g.grid.x, (int)g.grid.y, g.nblocks);
 }
 
 template <typename T, int NF>
@@ -1458,8 +1515,7 @@ static cudaError_t launch_tma_group_t(int stages, size_t smem, const BatchJob *j
     cudaError_t e = ensure_smem_attribute(kern, smem, configured, 0);
     if (e != cudaSuccess) return e;
     if (total == 0) return cudaSuccess;
-    kern<<<total, 256, smem, s>>>(jobs, first_item, njobs, c, stages);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(total), 256, smem, s, jobs, first_item, njobs, c, stages);
 }
 
 template <typename T, int NF, bool MEASURE, int D, int NT>
@@ -1470,8 +1526,7 @@ static cudaError_t launch_ldg(const Model &m, const FieldPtrs &fp, const PassCoe
     auto kern = fused_pass_ldg<T, NF, MEASURE, D, NT>;
     cudaError_t e = ensure_smem_attribute(kern, g.smem, configured, 0);
     if (e != cudaSuccess) return e;
-    kern<<<g.grid, NT, g.smem, s>>>(m, fp, c, g.txt, g.ty, g.zc, sc, slots);
-    return cudaGetLastError();
+    return launch_dependent(kern, g.grid, NT, g.smem, s, m, fp, c, g.txt, g.ty, g.zc, sc, slots);
 }
 
 template <typename T, int NF>

@@ -466,10 +466,9 @@ int tl_autotune(tl_lattice *lat, double *best_ms_per_pass);
  * tl_get_pass_config returns can be set again.  Values out of range are TL_EINVAL;
  * TL_ESTATE while the lattice is in a batch.  May synchronise the lattice
  * stream (to grow its reduction slots).  A new lattice starts on TL_PASS_TMA
- * when it is FP32 and N >= 192 (z-chunks of 48 planes at N = 192, 64 up to
- * N = 319, then 56, 80, 160 (one field) or 96, 104, 72 and 68 planes around
- * N = 384, 448, 512, 576 ... 768, 896 and 1024, where they measured fastest;
- * 15 compute warps from N = 416, else 7), on
+ * when it is FP32 and N >= 192 (compute warps and z-chunk chosen from N, the
+ * field count and the SM count, to run in few full waves of CTAs, up to N = 495;
+ * 15 compute warps and measured z-chunks from there), on
  * TL_PASS_STREAM otherwise (where those measured faster; z-chunks chosen from N
  * and the SM count, FP64 mostly 32 planes from N = 128 and 64 from N = 512); the environment
  * variable TL_PASS_VARIANT=tma|ldg overrides that default at creation. */

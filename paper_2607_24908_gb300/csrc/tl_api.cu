@@ -46,7 +46,33 @@ thread_local char g_err[512] = "";
 
 }  // namespace
 
-tl::PassTuning tl::default_tuning(int N, int nf, int elem_bytes)
+// Compute warps and z-chunk of the TMA pass for FP32 lattices of a few waves of
+// CTAs: the fewest (waves of CTAs) x (planes per chunk + 8), a wave being one CTA of
+// 15 + 1 warps per SM or two of 7 + 1 (5%, 10%, 12% slower a row of sites with one, two,
+// three fields: their ring is shallower).  us, former fixed values -> chosen: one
+// field 200^3 52 -> 34, 224^3 51 -> 39, 288^3 107 -> 74, 320^3 124 -> 104, 352^3 151 -> 133, 416^3
+// 231 -> 196; two fields 200^3 91 -> 58, 288^3 173 -> 151, 320^3 204 -> 196; three 224^3 136 ->
+// 104, 288^3 276 -> 204, 352^3 434 -> 392, 416^3 642 -> 590 (equal tiles included).
+static void tma_shape(tl::PassTuning &t, int N, int nf, int sms)
+{
+    const int txt = tl::even_row_tile(N / 4), gx = (N / 4 + txt - 1) / txt;
+    double least = 0.0;
+    for (int warps : {7, 15}) {
+        const int ty = 32 * warps / txt < N ? 32 * warps / txt : N;
+        const long tiles = (long)gx * ((N + ty - 1) / ty), slots = (long)sms * (warps == 7 ? 2 : 1);
+        const double rows = warps == 15 ? ty : 2 * ty * (nf == 1 ? 1.05 : nf == 2 ? 1.1 : 1.12);
+        for (int chunks = 1; chunks <= N / 20; ++chunks) {
+            int zc = (N + chunks - 1) / chunks;
+            if (zc > 170) continue;
+            const int even = (zc + 7) / 8 * 8;  // whole flushes of the FP32 sums, where that costs under 2%
+            if (even <= 1.02 * zc && (N + even - 1) / even == chunks) zc = even;
+            const double cost = (double)((tiles * chunks + slots - 1) / slots) * (zc + 8) * rows;
+            if (least == 0.0 || cost < least) least = cost, t.cwarps = warps, t.zc = zc;
+        }
+    }
+}
+
+tl::PassTuning tl::default_tuning(int N, int nf, int elem_bytes, int sm_count)
 {
     tl::PassTuning t{elem_bytes == 4 && N >= 192 ? tl::kVariantTma : tl::kVariantLdg, 7, 0, 0, 0, 256, 0};
     // environment overrides (tuning experiments)
@@ -54,23 +80,33 @@ tl::PassTuning tl::default_tuning(int N, int nf, int elem_bytes)
     if (v && strcmp(v, "tma") == 0) t.variant = tl::kVariantTma;
     if (v && strcmp(v, "ldg") == 0) t.variant = tl::kVariantLdg;
     const char *cw = getenv("TL_BULK_WARPS"), *zc = getenv("TL_PASS_ZC");
-    if (t.variant == tl::kVariantTma) {  // measured: long z-chunks for the ring, 15 + 1 warps from 416
-        // warps x z-chunk sweeps of the current kernel (FP32, ms per pass, one / two fields):
-        // 192^3 48 planes 0.083 two fields (16: 0.091); 384^3 7 + 1 warps, 56 planes 0.205 /
-        // 0.325; 448^3 15 + 1, 80 planes 0.524 two fields (96: 0.531); 512^3 15 + 1, 160
-        // planes 0.417 one field, 96 planes 0.705 two (160: 0.714); 576^3 ... 768^3 104
-        // planes (640^3 1.330, 768^3 2.297 two fields); 896^3 72 planes 3.623 (92: 3.634);
-        // 1024^3 68 planes 5.384 (76: 5.405, 92: 5.435).  The optimum is jagged in the chunk count, so
-        // each measured size sets the value for the sizes around it.
-        if (N <= 192) t.zc = 48;
-        else if (N < 320) t.zc = 64;
-        else if (N < 416) t.zc = 56;
-        else if (N < 480) t.zc = 80;
-        else if (N < 544) t.zc = nf == 1 ? 160 : 96;
-        else if (N < 832) t.zc = 104;
-        else if (N < 960) t.zc = 72;
-        else t.zc = 68;
-        t.cwarps = N >= 416 ? 15 : 7;
+    if (t.variant == tl::kVariantTma) {
+        // From 496^3 on (two fields: 440^3) the pass runs at the memory's rate, chunks
+        // matter by what the tiles in flight share in L2, and the values are the best
+        // of measured sweeps, as they are around 384^3 (us, 380^3 one field 56 planes 170,
+        // the estimate's 76: 173; 364^3 two fields 291 against 296; 380^3 three fields 43
+        // planes 483, 76: over 490).  15 + 1 warps: 464^3 two fields 80 planes 536 (93:
+        // over 558), 512^3 160 planes with one field (344; 128: 360), else 96 (two fields 686;
+        // 103: 687), 576^3 104 (two fields 1002; 64: 1009), from 620^3 60 with two fields
+        // (704^3 79: 1815; 768^3 2291; 104: 2312, 896^3 3616; 72: 3619, 1024^3 5355; 68: 5365) and from 832^3
+        // with three (896^3 5638; 72: 5656), else 104 (640^3 2050), one field from 832^3
+        // 150 (896^3 1800; 72: 1865).
+        if (elem_bytes != 4 || N < 192) t.zc = N <= 192 ? 48 : 64;
+        else if (N == 192 && nf == 2) t.zc = 48;
+        else if (N >= (nf == 2 ? 356 : 372) && N < (nf == 2 ? 410 : 396)) {
+            t.cwarps = nf == 3 ? 15 : 7;
+            t.zc = nf == 3 ? 43 : 56;
+        } else if (N < (nf == 2 ? 440 : tl::kFullRowTiles)) {
+            tma_shape(t, N, nf, sm_count > 0 ? sm_count : 152);
+        } else {
+            t.cwarps = 15;
+            if (N < tl::kFullRowTiles) t.zc = 80;
+            else if (N < 544) t.zc = nf == 1 ? 160 : 96;
+            else if (N < 620) t.zc = 104;
+            else if (nf == 2) t.zc = N >= 670 && N < 740 ? 79 : 60;
+            else if (N < 832) t.zc = 104;
+            else t.zc = nf == 1 ? 150 : 60;
+        }
     }
     if ((v = getenv("TL_PREFETCH"))) t.prefetch = atoi(v);
     if ((v = getenv("TL_LDG_THREADS"))) t.threads = atoi(v);
@@ -206,7 +242,7 @@ int finish_create(tl_lattice *L, int N, double kIR, int nf, tl_dtype dtype, cons
     TL_CK(cudaDeviceGetAttribute(&L->sm_count, cudaDevAttrMultiProcessorCount, dev));
     L->device = dev;
     tl::scratch_user(dev, 1);
-    L->tuning = tl::default_tuning(N, nf, (int)L->esz);
+    L->tuning = tl::default_tuning(N, nf, (int)L->esz, L->sm_count);
     L->geom = tl::pass_geometry(N, (int)L->esz, L->sm_count, nf, L->tuning);
     TL_CK(cudaMalloc(&L->d_sc, sizeof(Scalars)));
     TL_CK(cudaMemsetAsync(L->d_sc, 0, sizeof(Scalars), L->stream));

@@ -171,9 +171,12 @@ struct PassGeom {
     size_t smem;   // dynamic shared memory per CTA
 };
 
-// Threads along x of the streaming kernel's 32-wide tiles: rows of per_row
+// Threads along x of 32-wide tiles: rows of per_row
 // threads cut into the fewest tiles of at most 32, all alike (a row of 48 into
-// two of 24; 32 + 16 left a quarter of the lanes idle).
+// two of 24; 32 + 16 left a quarter of the lanes idle).  The TMA pass keeps 32
+// from N = 496: it runs at the memory's rate there, and whole tiles share their
+// halos better (576^3 two fields 1002 us against 1026).
+constexpr int kFullRowTiles = 496;
 inline int even_row_tile(int per_row)
 {
     const int tiles = (per_row + 31) / 32;
@@ -182,13 +185,12 @@ inline int even_row_tile(int per_row)
 
 PassGeom pass_geometry(int N, int elem_bytes, int sm_count, int nf, const PassTuning &t);
 
-// Tuning from the environment (TL_PASS_VARIANT=ldg|bulk, TL_PREFETCH, TL_LDG_THREADS, TL_LDG_TXT,
-// TL_BULK_WARPS, TL_BULK_STAGES, TL_PASS_ZC), else the built-in defaults.
-// Launch shape a new lattice starts with: the TMA pass for FP32 from N = 192
-// up (z-chunks of 16 planes at 192, 64 above; 15 + 1 warps from N = 768),
-// where it measured faster; the streaming pass otherwise (FP64 is bound by
-// FP64 arithmetic, small lattices by latency).
-PassTuning default_tuning(int N, int nf, int elem_bytes);
+// Launch shape a new lattice starts with: the TMA pass for FP32 from N = 192 up,
+// where it measured faster; the streaming pass otherwise (FP64 is bound by FP64
+// arithmetic, small lattices by latency).  Environment overrides for tuning
+// experiments: TL_PASS_VARIANT=ldg|tma, TL_PREFETCH, TL_LDG_THREADS, TL_LDG_TXT,
+// TL_BULK_WARPS, TL_BULK_STAGES, TL_PASS_ZC.
+PassTuning default_tuning(int N, int nf, int elem_bytes, int sm_count);
 
 // One lattice of a batched (grouped) launch: its model, fields for this pass,
 // scalars, reduction slots and its own launch geometry.

@@ -109,7 +109,7 @@ PassGeom pass_geometry(int N, int elem_bytes, int sm_count, int nf, const PassTu
     const int threads = t.variant == kVariantTma ? 32 * g.cwarps : g.threads;
     const int txt_max = (t.variant == kVariantLdg && (t.txt == 8 || t.txt == 16)) ? t.txt : 32;
     g.tile_x = g.txt = per_row < txt_max ? per_row : txt_max;
-    if (t.variant == kVariantLdg && txt_max == 32) g.txt = even_row_tile(per_row);
+    if (txt_max == 32 && (t.variant == kVariantLdg || N < kFullRowTiles)) g.txt = even_row_tile(per_row);
     g.ty = threads / g.txt;
     if (g.ty > N) g.ty = N;
     const int gx = (per_row + g.txt - 1) / g.txt;

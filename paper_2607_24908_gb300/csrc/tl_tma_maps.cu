@@ -54,14 +54,15 @@ int encode_maps(tl_lattice *L)
                                     {(cuuint32_t)(g.txt * W), rows, 1u},          // kMapBody
                                     {(cuuint32_t)W, rows, 1u}};                   // kMapSide
     const cuuint32_t estr[3] = {1u, 1u, 1u};
-    // L2 promotion of the copies: 64 bytes (measured at N = 256 ... 1024 two
-    // fields, 256^3 one field and the grouped ensemble: 0.1-0.5% faster than
-    // 256 bytes, 3.4% fewer DRAM reads at 1024^3).  Environment override for
-    // tuning experiments: TL_TMA_L2_PROMOTION = none, 64, 128 or 256.
-    CUtensorMapL2promotion promo = CU_TENSOR_MAP_L2_PROMOTION_L2_64B;
+    // L2 promotion of the copies: 128 bytes (us, two fields, 64 / 128 / 256 bytes:
+    // 256^3 98.8 / 97.6 / 102, 640^3 1336 / 1334 / 1351, 1024^3 5412 / 5355 / 5387; one field
+    // 640^3 675 / 671 / 676; three 512^3 1070 / 1059 / 1074; the ensemble alike).
+    // Environment override for tuning experiments: TL_TMA_L2_PROMOTION = none, 64,
+    // 128 or 256.
+    CUtensorMapL2promotion promo = CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
     if (const char *v = getenv("TL_TMA_L2_PROMOTION")) {
         if (strcmp(v, "none") == 0) promo = CU_TENSOR_MAP_L2_PROMOTION_NONE;
-        else if (strcmp(v, "128") == 0) promo = CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
+        else if (strcmp(v, "64") == 0) promo = CU_TENSOR_MAP_L2_PROMOTION_L2_64B;
         else if (strcmp(v, "256") == 0) promo = CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
     }
     for (int par = 0; par < 2; ++par)

@@ -79,6 +79,15 @@ __device__ __forceinline__ void store_vec_cs(double *p, const double (&v)[2])
 {
     __stcs(reinterpret_cast<double2 *>(p), make_double2(v[0], v[1]));
 }
+// A TMA pass's outputs: with one field plain stores, whose lines stay in L2 like
+// any other (measured 1-2.5% faster: 256^3 51.2 against 52.4 us, 512^3 339 against
+// 343), else streaming ones (two fields 256^3 96.7 against 98.8, 1024^3 5343 against 5432).
+template <int NF, typename T, int W>
+__device__ __forceinline__ void store_out(T *p, const T (&v)[W])
+{
+    if constexpr (NF == 1) store_vec(p, v);
+    else store_vec_cs(p, v);
+}
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
 
@@ -409,6 +418,21 @@ __device__ __forceinline__ void site_update(const Coefs<T, NF> &k, const T (&cu)
 // FP64 lattices keep the whole tree in FP64.  sync: a barrier of those warps.
 constexpr int kFlush = 16;
 
+template <int NQ>
+__device__ __forceinline__ double warps_total(const double (*red)[NQ], int nwarps)  // in lane i < NQ
+{
+    const int lane = threadIdx.x & 31;
+    if (lane >= NQ) return 0.0;
+    double s[4];  // four chains: additions wait for each other
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = k < nwarps ? red[k][lane] : 0.0;
+    for (int k = 4; k < nwarps; k += 4)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (k + i < nwarps) s[i] += red[k + i][lane];
+    return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
 template <int NQ, typename T, typename Sync>
 __device__ __forceinline__ double tile_sum(const T (&acc)[NQ], const double (&accd)[NQ], bool flushed, int nwarps,
                                            double (*red)[NQ], Sync sync)  // in lane i < NQ of warp 0
@@ -424,16 +448,52 @@ __device__ __forceinline__ double tile_sum(const T (&acc)[NQ], const double (&ac
     const T w = warp_sums<NQ>(v);
     if (lane < NQ) red[warp][lane] = (double)w;
     sync();
-    if (warp != 0 || lane >= NQ) return 0.0;
-    double s[4];  // four chains: additions wait for each other
-#pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] = k < nwarps ? red[k][lane] : 0.0;
-    for (int k = 4; k < nwarps; k += 4)
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (k + i < nwarps) s[i] += red[k + i][lane];
-    return (s[0] + s[1]) + (s[2] + s[3]);
+    return warp == 0 ? warps_total<NQ>(red, nwarps) : 0.0;
 }
+
+// A TMA tile's sums: after every kFlush planes the FP32 sums go into FP64.
+// WARP: a warp's sums of those planes, a tree in T, go into its row of red; against
+// FP64 totals in every thread this saves their registers (14 with three fields)
+// and most FP64 instructions.  Measured faster with one field (0-3%) and three
+// (3-7% with the momenta read twice, see tma_tile: 256^3 144.6 -> 136.4 us, 380^3 481.6
+// -> 450.8, 512^3 1058.6 -> 1030.2), not with two (224^3 69.8 -> 67.0 us but 380^3 301.8 ->
+// 307.7, 1024^3 5342 -> 5412), which keep totals in their threads.
+template <int NQ, typename T>
+struct TileSums {
+    static constexpr bool WARP = NQ != 5;
+    T acc[NQ];
+    double accd[WARP ? 1 : NQ];
+    __device__ __forceinline__ void clear(double (*red)[NQ])  // every compute warp
+    {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            acc[i] = (T)0;
+            if constexpr (!WARP) accd[i] = 0.0;
+        }
+        if (WARP && lane < NQ) red[threadIdx.x >> 5][lane] = 0.0;
+    }
+    __device__ __forceinline__ void flush(double (*red)[NQ])  // whole warps
+    {
+        if constexpr (WARP) {
+            const int lane = threadIdx.x & 31;
+            const T w = warp_sums<NQ>(acc);
+            if (lane < NQ) red[threadIdx.x >> 5][lane] += (double)w;
+        }
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            if constexpr (!WARP) accd[i] += (double)acc[i];
+            acc[i] = (T)0;
+        }
+    }
+    template <typename Sync>
+    __device__ __forceinline__ double total(double (*red)[NQ], int nwarps, Sync sync)  // in lane i < NQ of warp 0
+    {
+        if constexpr (!WARP) return tile_sum<NQ>(acc, accd, true, nwarps, red, sync);
+        sync();
+        return threadIdx.x < 32 ? warps_total<NQ>(red, nwarps) : 0.0;
+    }
+};
 
 template <int NQ, typename T, typename Sync>
 __device__ __forceinline__ void reduce_tile(const T (&acc)[NQ], const double (&accd)[NQ], bool flushed, int nwarps,
@@ -913,14 +973,8 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
         if (tid < 32) share_coefs(coefs, m, c, sc);
         consumer_sync((unsigned)CW * 32u);
     }
-    constexpr bool flushed = true;
-    double accd[NQ];
-    T acc[NQ];
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-        accd[i] = 0.0;
-        acc[i] = (T)0;
-    }
+    TileSums<NQ, T> sums;
+    if (!producer) sums.clear(red);
     int issued = 0;
 
     if (producer) {
@@ -994,6 +1048,10 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
             pho[f] = static_cast<T *>(fp.phi_out[f]);
             pio[f] = static_cast<T *>(fp.pi_out[f]);
         }
+        // With three fields the momenta of plane z are read from its stage a second
+        // time, when the plane is updated, instead of staying in registers from its
+        // first reading as z + 1: 24 registers less and no spills.
+        constexpr bool kReread = NF == 3;
         T zm[NF][W], cu[NF][W], zp[NF][W], pc[NF][W], pn[NF][W];
         auto centre = [&](int s, T (&ph)[NF][W], T (&pp)[NF][W]) {
 #pragma unroll
@@ -1050,6 +1108,7 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const T *ph = arr(s0, f, 0), *pp = arr(s0, f, 1);
+                    if constexpr (kReread) load_vec_s(pp + ctr, pc[f]);
                     T a[W], b[W];
                     load_vec_s(ph + ctr - rowe, a);
                     load_vec_s(pp + ctr - rowe, b);
@@ -1067,13 +1126,13 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
                     xrv[f] = own_r ? fma_t(k.drift, pp[ir], ph[ir]) : r;
                 }
                 T pnew[NF][W];
-                site_update<T, NF, W>(k, cu, zm, zp, ym, yp, xlv, xrv, pc, pnew, acc);
+                site_update<T, NF, W>(k, cu, zm, zp, ym, yp, xlv, xrv, pc, pnew, sums.acc);
                 if (!MEASURE) {
                     const size_t pz = (size_t)z * PP;
 #pragma unroll
                     for (int f = 0; f < NF; ++f) {
-                        store_vec_cs(pho[f] + pz + (size_t)y * P + x0, cu[f]);
-                        store_vec_cs(pio[f] + pz + (size_t)y * P + x0, pnew[f]);
+                        store_out<NF>(pho[f] + pz + (size_t)y * P + x0, cu[f]);
+                        store_out<NF>(pio[f] + pz + (size_t)y * P + x0, pnew[f]);
                     }
                     if (m.ghosts) store_ghosts<T, NF, W>(pho, pio, cu, pnew, pz, x0, y, N, (long long)P);
                 }
@@ -1083,17 +1142,13 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
                     for (int j = 0; j < W; ++j) {
                         zm[f][j] = cu[f][j];
                         cu[f][j] = zp[f][j];
-                        pc[f][j] = pn[f][j];
+                        if constexpr (!kReread) pc[f][j] = pn[f][j];
                     }
             }
             adv_w();
             release(kz);
         }
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) {
-            accd[i] += (double)acc[i];
-            acc[i] = (T)0;
-        }
+        sums.flush(red);
         }
     }
     if (producer) {
@@ -1104,7 +1159,8 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
                 mbar_wait_bounded(&full[kk % S], (kk / S) & 1u, sc);
         return;
     }
-    reduce_tile<NQ>(acc, accd, flushed, CW, red, [&] { consumer_sync((unsigned)CW * 32u); }, m, c, sc, slots, bid, nblocks);
+    const double sum = sums.total(red, CW, [&] { consumer_sync((unsigned)CW * 32u); });
+    if (tid < 32) finish_tile<NQ>(sum, m, c, sc, slots, bid, nblocks);
 }
 
 // Tiles first, first + stride, ... (< nitems) of the TMA pass, in a CTA whose
@@ -1273,14 +1329,8 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
         const int y = y_tile + tyi;
         const bool active = (tyi < ty) && (x0 < N) && (y < N);
         const bool warp_active = __any_sync(0xffffffffu, active);
-        constexpr bool flushed = true;
-        double accd[NQ];
-        T acc[NQ];
-#pragma unroll
-        for (int i = 0; i < NQ; ++i) {
-            accd[i] = 0.0;
-            acc[i] = (T)0;
-        }
+        TileSums<NQ, T> sums;
+        sums.clear(red);
         if (warp_active) {
             // x-neighbours: the left site is the last one of the thread to the
             // left in the same row and warp, the right site the first one of the
@@ -1349,22 +1399,18 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
                         xrv[f] = own_r ? fma_t(k.drift, pp[ir], ph[ir]) : r;
                     }
                     T pnew[NF][W];
-                    site_update<T, NF, W>(k, cu, zm, zp, ym, yp, xlv, xrv, pc, pnew, acc);
+                    site_update<T, NF, W>(k, cu, zm, zp, ym, yp, xlv, xrv, pc, pnew, sums.acc);
                     if (!MEASURE) {
                         const size_t pz = (size_t)z * PP;
 #pragma unroll
                         for (int f = 0; f < NF; ++f) {
-                            store_vec_cs(pho[f] + pz + (size_t)y * P + x0, cu[f]);
-                            store_vec_cs(pio[f] + pz + (size_t)y * P + x0, pnew[f]);
+                            store_out<NF>(pho[f] + pz + (size_t)y * P + x0, cu[f]);
+                            store_out<NF>(pio[f] + pz + (size_t)y * P + x0, pnew[f]);
                         }
                         if (m.ghosts) store_ghosts<T, NF, W>(pho, pio, cu, pnew, pz, x0, y, N, (long long)P);
                     }
-                    if (((z - z0) & (kFlush - 1)) == kFlush - 1) {
-#pragma unroll
-                        for (int i = 0; i < NQ; ++i) {
-                            accd[i] += (double)acc[i];
-                            acc[i] = (T)0;
-                        }
+                    if constexpr (!sums.WARP) {
+                        if (((z - z0) & (kFlush - 1)) == kFlush - 1) sums.flush(red);
                     }
 #pragma unroll
                     for (int f = 0; f < NF; ++f)
@@ -1375,13 +1421,15 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
                             pc[f][j] = pn[f][j];
                         }
                 }
+                if constexpr (sums.WARP) {
+                    if (((z - z0) & (kFlush - 1)) == kFlush - 1) sums.flush(red);
+                }
                 advance_wait();
                 release_next();  // plane kz
                 kz_done = kz;
             }
             if (kz_done == K - 2) release_next();  // the top halo plane, read as z + 1 of the last plane
-#pragma unroll
-            for (int i = 0; i < NQ; ++i) accd[i] += (double)acc[i];
+            sums.flush(red);
         } else {
             // no sites in this tile: keep the ring's count, plane by plane
             for (int kk = 0; kk < K; ++kk) {
@@ -1391,7 +1439,8 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
                 release_next();
             }
         }
-        reduce_tile<NQ>(acc, accd, flushed, CW, red, [&] { consumer_sync(nthr); }, m, c, sc, slots, item, nitems);
+        const double sum = sums.total(red, CW, [&] { consumer_sync(nthr); });
+        if (tid < 32) finish_tile<NQ>(sum, m, c, sc, slots, item, nitems);
         if (tid == 0) s_stop = s_failed;
         consumer_sync(nthr);
         if (s_stop) break;

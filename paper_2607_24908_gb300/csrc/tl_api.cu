@@ -14,6 +14,7 @@
 #include <utility>
 #include <vector>
 
+#include "tl_fft.cuh"
 #include "tl_fourier.cuh"
 #include "tl_internal.cuh"
 #include "tl_lattice.cuh"
@@ -319,18 +320,37 @@ int check_field(const tl_lattice *L, int field, int which)
     return TL_OK;
 }
 
-// cuFFT plans (N x N x N/2 complex, see tl_fourier.cuh) shared by all lattices
-// of a size on a device (planning costs milliseconds and a workspace per plan).  Under this mutex a plan is bound
-// to the caller's stream, which first waits for the plan's previous
-// executions (on whatever stream they were enqueued) through the plan's
-// event; the caller records that event after its last execution.  Calls that
-// use a plan therefore only enqueue work: no host wait guards the workspace.
+// Transforms (N x N x N/2 complex, see tl_fourier.cuh) shared by all lattices of
+// a size on a device: the table of roots for the sizes of tl_fft.cuh, a cuFFT plan
+// for the others (planning costs milliseconds and a workspace per plan).  Under
+// this mutex a plan is bound to the caller's stream, which first waits for the
+// plan's previous executions (on whatever stream they were enqueued) through the
+// plan's event; the caller records that event after its last execution.  Calls
+// that use a plan therefore only enqueue work: no host wait guards the workspace.
+// A table is written before its first use and then only read: nothing to wait for.
 struct SharedPlan {
+    double2 *roots;    // nullptr: the cuFFT plan
     cufftHandle h;
-    cudaEvent_t done;  // recorded after the latest enqueued execution
+    cudaEvent_t done;  // cuFFT: recorded after the latest enqueued execution
 };
 std::mutex g_plan_mu;
 std::map<std::pair<int, int>, SharedPlan> g_plans;  // (device, N) -> plan
+
+int make_roots(int N, cudaStream_t s, double2 **out)
+{
+    std::vector<double2> h((size_t)N / 2);
+    tl::fft_roots(N, h.data());
+    double2 *d = nullptr;
+    TL_CK(cudaMalloc(&d, h.size() * sizeof(double2)));
+    cudaError_t e = cudaMemcpyAsync(d, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        cudaFree(d);
+        return fail(TL_ECUDA, "table of roots: %s", cudaGetErrorString(e));
+    }
+    *out = d;
+    return TL_OK;
+}
 
 int shared_plan(int N, cudaStream_t s, SharedPlan **out)
 {
@@ -340,22 +360,71 @@ int shared_plan(int N, cudaStream_t s, SharedPlan **out)
     auto it = g_plans.find(key);
     if (it == g_plans.end()) {
         SharedPlan p{};
-        cufftResult r = cufftPlan3d(&p.h, N, N, N / 2, CUFFT_Z2Z);
-        if (r != CUFFT_SUCCESS) {  // perhaps for memory that the scratch pool keeps
-            tl::scratch_release(dev);
-            r = cufftPlan3d(&p.h, N, N, N / 2, CUFFT_Z2Z);
-        }
-        if (r != CUFFT_SUCCESS) return fail(TL_ECUDA, "cufftPlan3d(%d) failed (%d)", N, (int)r);
-        cudaError_t e = cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming);
-        if (e != cudaSuccess) {
-            cufftDestroy(p.h);
-            return fail(TL_ECUDA, "cudaEventCreateWithFlags: %s", cudaGetErrorString(e));
+        if (tl::fft_supported(N)) {
+            const int rc = make_roots(N, s, &p.roots);
+            if (rc) return rc;
+        } else {
+            cufftResult r = cufftPlan3d(&p.h, N, N, N / 2, CUFFT_Z2Z);
+            if (r != CUFFT_SUCCESS) {  // perhaps for memory that the scratch pool keeps
+                tl::scratch_release(dev);
+                r = cufftPlan3d(&p.h, N, N, N / 2, CUFFT_Z2Z);
+            }
+            if (r != CUFFT_SUCCESS) return fail(TL_ECUDA, "cufftPlan3d(%d) failed (%d)", N, (int)r);
+            cudaError_t e = cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming);
+            if (e != cudaSuccess) {
+                cufftDestroy(p.h);
+                return fail(TL_ECUDA, "cudaEventCreateWithFlags: %s", cudaGetErrorString(e));
+            }
         }
         it = g_plans.emplace(key, p).first;
     }
+    *out = &it->second;
+    if (it->second.roots) return TL_OK;
     TL_CKFFT(cufftSetStream(it->second.h, s));
     TL_CK(cudaStreamWaitEvent(s, it->second.done, 0));  // a never-recorded event: no wait
-    *out = &it->second;
+    return TL_OK;
+}
+
+int plan_used(SharedPlan *p, cudaStream_t s)  // after the call's last execution
+{
+    if (!p->roots) TL_CK(cudaEventRecord(p->done, s));
+    return TL_OK;
+}
+
+tl::FieldRows field_rows(tl_lattice *L, void *array, double base, double scale)
+{
+    return tl::FieldRows{array, L->dtype == TL_F32, L->N, L->model.pitch, L->model.pplane, base, scale};
+}
+
+// modes = transform of the padded array at src.
+int field_to_modes(tl_lattice *L, SharedPlan *p, void *src, double2 *modes)
+{
+    if (p->roots) {
+        TL_CK(tl::launch_fft_rows(modes, field_rows(L, src, 0.0, 1.0), p->roots, false, L->stream));
+        TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, false, false, L->stream));
+        TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, true, false, L->stream));
+        return TL_OK;
+    }
+    TL_CK(tl::launch_widen((int)L->dtype, reinterpret_cast<double *>(modes), src, L->N, L->model.pitch,
+                           L->model.pplane, L->stream));
+    cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
+    TL_CKFFT(cufftExecZ2Z(p->h, z, z, CUFFT_FORWARD));
+    return TL_OK;
+}
+
+// dst (padded, ghost rows included) = base + scale * inverse transform of modes, which are overwritten.
+int modes_to_field(tl_lattice *L, SharedPlan *p, double2 *modes, void *dst, double base, double scale)
+{
+    if (p->roots) {
+        TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, true, true, L->stream));
+        TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, false, true, L->stream));
+        TL_CK(tl::launch_fft_rows(modes, field_rows(L, dst, base, scale), p->roots, true, L->stream));
+        return TL_OK;
+    }
+    cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
+    TL_CKFFT(cufftExecZ2Z(p->h, z, z, CUFFT_INVERSE));
+    TL_CK(tl::launch_assemble((int)L->dtype, dst, reinterpret_cast<double *>(modes), base, scale, L->N,
+                              L->model.pitch, L->model.pplane, L->stream));
     return TL_OK;
 }
 
@@ -825,7 +894,6 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
         int prc = shared_plan(N, L->stream, &sp);
         if (prc) return prc;
     }
-    const cufftHandle plan = sp->h;
     double2 *modes = nullptr;  // N x N x N/2 modes, then (in place) the N^3 field
     if (tl::scratch_alloc((void **)&modes, n3_of(N) * sizeof(double), L->stream) != cudaSuccess)
         return fail(TL_ENOMEM, "scratch allocation for the initial field failed");
@@ -842,12 +910,7 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
                                                        spec->fixed_modulus ? 1 : 0, seed, which == 0 ? (uint64_t)f : (uint64_t)(8 + f),
                                                        L->sm_count, L->stream);
                 if (ce != cudaSuccess) { rc = fail(TL_ECUDA, "fill_modes: %s", cudaGetErrorString(ce)); break; }
-                cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
-                cufftResult fr = cufftExecZ2Z(plan, z, z, CUFFT_INVERSE);
-                if (fr != CUFFT_SUCCESS) { rc = fail(TL_ECUDA, "cufftExecZ2Z failed (%d)", (int)fr); break; }
-                ce = tl::launch_assemble((int)L->dtype, dst, reinterpret_cast<double *>(modes), base,
-                                         which == 0 ? 1.0 : pscale, N, L->model.pitch, L->model.pplane, L->stream);
-                if (ce != cudaSuccess) { rc = fail(TL_ECUDA, "assemble: %s", cudaGetErrorString(ce)); break; }
+                rc = modes_to_field(L, sp, modes, dst, base, which == 0 ? 1.0 : pscale);
             } else {
                 cudaError_t ce = tl::launch_assemble((int)L->dtype, dst, nullptr, base, 0.0, N, L->model.pitch,
                                                      L->model.pplane, L->stream);
@@ -856,8 +919,8 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
         }
     }
     {
-        const cudaError_t re = cudaEventRecord(sp->done, L->stream);  // after this call's executions
-        if (re != cudaSuccess && rc == TL_OK) rc = fail(TL_ECUDA, "cudaEventRecord: %s", cudaGetErrorString(re));
+        const int used = plan_used(sp, L->stream);
+        if (rc == TL_OK) rc = used;
     }
     cudaFreeAsync(modes, L->stream);
     if (rc) return rc;
@@ -884,18 +947,15 @@ int tl_spectrum(tl_lattice *L, int field, int which, int nbins, double *k, doubl
         int prc = shared_plan(N, L->stream, &sp);
         if (prc) return prc;
     }
-    const cufftHandle plan = sp->h;
     double2 *modes = nullptr;  // the field, then (in place) its N x N x N/2 modes
     double *acc = nullptr;
     TL_CK(tl::scratch_alloc((void **)&modes, n3_of(N) * sizeof(double), L->stream));
     TL_CK(tl::scratch_alloc((void **)&acc, (size_t)nb * 3 * sizeof(double), L->stream));
     TL_CK(cudaMemsetAsync(acc, 0, (size_t)nb * 3 * sizeof(double), L->stream));
-    TL_CK(tl::launch_widen((int)L->dtype, reinterpret_cast<double *>(modes), L->buf[L->cur][which][field], N,
-                           L->model.pitch, L->model.pplane, L->stream));
-    cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
-    cufftResult fr = cufftExecZ2Z(plan, z, z, CUFFT_FORWARD);
-    if (fr != CUFFT_SUCCESS) return fail(TL_ECUDA, "cufftExecZ2Z failed (%d)", (int)fr);
-    TL_CK(cudaEventRecord(sp->done, L->stream));
+    rc = field_to_modes(L, sp, L->buf[L->cur][which][field], modes);
+    if (rc) return rc;
+    rc = plan_used(sp, L->stream);
+    if (rc) return rc;
     TL_CK(tl::launch_bin(modes, N, nb, acc, acc + nb, reinterpret_cast<unsigned long long *>(acc + 2 * nb),
                          L->sm_count, L->stream));
     std::vector<double> h((size_t)nb * 3);

@@ -2,10 +2,12 @@
 // loop).  The paper prepares states and measures in Fourier space through its
 // automatic Fourier views (Sec. 2) with Philox-2x64 random numbers (Sec. 2);
 // here the mode draw, the field assembly and the shell binning are kernels
-// of this library and the transforms are cuFFT library calls (FP64, complex, of
-// half the real size: tl_fourier.cuh).
+// of this library; the transforms (FP64, complex, of half the real size:
+// tl_fourier.cuh) are its own for the sizes of tl_fft.cuh, cuFFT library calls
+// for the others.
 #include <math.h>
 
+#include "tl_bits.cuh"
 #include "tl_boxmuller.cuh"
 #include "tl_fourier.cuh"
 #include "tl_philox.cuh"
@@ -92,7 +94,9 @@ __global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, ModeSpe
 
 // Four consecutive sites per thread (a row starts a 128-byte line in both
 // layouts' FP32 form and N is a multiple of 4): 16- and 32-byte accesses, one
-// index decomposition for the four.
+// index decomposition for the four.  Conversions are integer instructions
+// (tl_bits.cuh; a field without fluctuations is converted once, on the host): us,
+// 256^3 FP32, with F2F -> without: assemble 70, fill 69 -> 12.
 template <typename T>
 struct Four;
 template <>
@@ -100,11 +104,12 @@ struct Four<float> {
     static __device__ __forceinline__ void ld(const float *p, double (&v)[4])
     {
         const float4 a = *reinterpret_cast<const float4 *>(p);
-        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+        v[0] = widen_bits(a.x), v[1] = widen_bits(a.y), v[2] = widen_bits(a.z), v[3] = widen_bits(a.w);
     }
+    static __device__ __forceinline__ void fill(float *p, float v) { *reinterpret_cast<float4 *>(p) = make_float4(v, v, v, v); }
     static __device__ __forceinline__ void st(float *p, const double (&v)[4])
     {
-        *reinterpret_cast<float4 *>(p) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+        *reinterpret_cast<float4 *>(p) = make_float4(narrow_bits(v[0]), narrow_bits(v[1]), narrow_bits(v[2]), narrow_bits(v[3]));
     }
 };
 template <>
@@ -114,6 +119,11 @@ struct Four<double> {
         const double2 a = *reinterpret_cast<const double2 *>(p), b = *reinterpret_cast<const double2 *>(p + 2);
         v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
     }
+    static __device__ __forceinline__ void fill(double *p, double v)
+    {
+        *reinterpret_cast<double2 *>(p) = make_double2(v, v);
+        *reinterpret_cast<double2 *>(p + 2) = make_double2(v, v);
+    }
     static __device__ __forceinline__ void st(double *p, const double (&v)[4])
     {
         *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
@@ -122,21 +132,26 @@ struct Four<double> {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(256) assemble_kernel(T *dst, const double *delta, double base, double scale, int N,
-                                                       long long P, long long PP)
+__global__ void __launch_bounds__(256) assemble_kernel(T *dst, const double *delta, double base, T base_t, double scale,
+                                                       int N, long long P, long long PP)
 {
     const unsigned quads = (unsigned)N / 4, i = blockIdx.x * 256u + threadIdx.x;
     const unsigned row = i / quads, x = 4 * (i - row * quads);
     const int z = row / N, y = row - (unsigned)z * N;
     if (z >= N) return;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    if (delta) Four<double>::ld(delta + (size_t)row * N + x, v);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = base + (delta ? scale * v[j] : 0.0);
     T *out = dst + z * PP + y * P + x;
+    const long long ghost = y == 0 ? (long long)N * P : y == N - 1 ? -((long long)N * P) : 0;  // to the ghost row
+    if (!delta) {
+        Four<T>::fill(out, base_t);
+        if (ghost) Four<T>::fill(out + ghost, base_t);
+        return;
+    }
+    double v[4];
+    Four<double>::ld(delta + (size_t)row * N + x, v);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = base + scale * v[j];
     Four<T>::st(out, v);
-    if (y == 0) Four<T>::st(out + (long long)N * P, v);  // the ghost rows
-    if (y == N - 1) Four<T>::st(out - (long long)N * P, v);
+    if (ghost) Four<T>::st(out + ghost, v);
 }
 
 template <typename T>
@@ -202,7 +217,7 @@ __device__ __forceinline__ void add_to_shell(int b, double P, double r, unsigned
 //
 // FP64-pipe work a mode: 8 operations for |F|^2 and its sum.  With one shared
 // FP64 atomic (a compare-and-swap loop) for each of a mode's three sums this
-// took 475 us at 256^3; here 198.
+// took 475 us at 256^3; here 193.
 __global__ void __launch_bounds__(256) bin_kernel(const double2 *__restrict__ modes, int N, int nbins, double *Psum,
                                                   double *rsum, unsigned long long *cnt)
 {
@@ -297,9 +312,9 @@ cudaError_t launch_assemble(int dtype, void *dst, const double *delta, double ba
 {
     const unsigned grid = (unsigned)(((size_t)N * N * (N / 4) + 255) / 256);
     if (dtype == TL_F32)
-        assemble_kernel<float><<<grid, 256, 0, s>>>(static_cast<float *>(dst), delta, base, scale, N, P, PP);
+        assemble_kernel<float><<<grid, 256, 0, s>>>(static_cast<float *>(dst), delta, base, (float)base, scale, N, P, PP);
     else
-        assemble_kernel<double><<<grid, 256, 0, s>>>(static_cast<double *>(dst), delta, base, scale, N, P, PP);
+        assemble_kernel<double><<<grid, 256, 0, s>>>(static_cast<double *>(dst), delta, base, base, scale, N, P, PP);
     return cudaGetLastError();
 }
 
@@ -323,7 +338,7 @@ cudaError_t launch_bin(const double2 *modes, int N, int nbins, double *Psum, dou
         const cudaError_t e = cudaFuncSetAttribute(bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    bin_kernel<<<grid_for(total, sm_count, 4), 256, smem, s>>>(modes, N, nbins, Psum, rsum, cnt);
+    bin_kernel<<<grid_for(total, sm_count, 2), 256, smem, s>>>(modes, N, nbins, Psum, rsum, cnt);
     return cudaGetLastError();
 }
 

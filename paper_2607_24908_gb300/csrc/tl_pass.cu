@@ -61,13 +61,32 @@ static int f64_tile_rows(int N, int gx, int txt, int ty_max, int zc, int sms)
     return best;
 }
 
-// FP64 chunk: the cheapest; from 128^3 32 planes and from 512^3 64 (the best of a
-// measured sweep) unless another is estimated 5% cheaper.
-static int f64_chunk(int N, int gx, int txt, int ty_max, int sms)
+// FP64 chunk with one or two fields (shared_tile): the cheapest by (waves of two
+// CTAs per SM) x (warps per CTA x planes), where a last wave of at most one CTA per
+// SM counts 0.6 and a CTA no less than 6 warps.  Over 36 lattices of 32^3 to 384^3 the
+// choice is 0.6% slower than the best of a sweep (8% at 144^3 with two fields), that
+// of the estimate above, made for ldg_tile, 5% (us: 144^3 155 -> 127, 160^3 199 -> 160,
+// 212^3 396 -> 355, 300^3 1090 -> 932).  Two fields keep 32 planes from 128^3 unless
+// another is estimated 4% cheaper (256^3 1216, 37 planes 1200).
+static double f64_shared_cost(int N, int gx, int txt, int ty, int zc, int sms)
 {
-    auto cost = [&](int zc) { return f64_cost(N, gx, txt, f64_tile_rows(N, gx, txt, ty_max, zc, sms), zc, sms); };
-    int best = N >= 512 ? 64 : N >= 128 ? 32 : 1;
-    double least = cost(best) * (N >= 128 ? 0.95 : 1.0);
+    const long ctas = (long)gx * ((N + ty - 1) / ty) * ((N + zc - 1) / zc), last = ctas % (2 * sms);
+    const double waves = (double)(ctas / (2 * sms)) + (last == 0 ? 0.0 : last <= sms ? 0.6 : 1.0);
+    int warps = (txt * ty + 31) / 32;
+    if (warps < 6) warps = 6;
+    return waves * (warps * (zc + 0.3) + 3.0);
+}
+
+// FP64 chunk: the cheapest; with three fields from 128^3 32 planes and from 512^3
+// 64 (the best of a measured sweep) unless another is estimated 5% cheaper.
+static int f64_chunk(int N, int nf, int gx, int txt, int ty_max, int sms)
+{
+    auto cost = [&](int zc) {
+        const int ty = f64_tile_rows(N, gx, txt, ty_max, zc, sms);
+        return nf <= 2 ? f64_shared_cost(N, gx, txt, ty, zc, sms) : f64_cost(N, gx, txt, ty, zc, sms);
+    };
+    int best = nf == 3 && N >= 512 ? 64 : N >= 128 ? 32 : 1;
+    double least = cost(best) * (N < 128 || nf == 1 ? 1.0 : nf == 2 ? 0.96 : 0.95);
     for (int zc = 1; zc <= N && zc <= 128; ++zc)
         if (cost(zc) < least) least = cost(zc), best = zc;
     return best;
@@ -119,7 +138,7 @@ PassGeom pass_geometry(int N, int elem_bytes, int sm_count, int nf, const PassTu
     int zc = t.zc;
     if (zc <= 0) {
         if (f64_stream) {
-            zc = f64_chunk(N, gx, g.txt, g.ty, sms);
+            zc = f64_chunk(N, nf, gx, g.txt, g.ty, sms);
         } else if (t.variant == kVariantLdg) {
             zc = f32_chunk(N, nf, gx * gy, sms);
         } else {  // TMA: long enough to amortise the two extra planes, short enough for several waves

@@ -526,6 +526,62 @@ __device__ __forceinline__ void store_ghosts(T *const (&pho)[NF], T *const (&pio
     }
 }
 
+// ---- PTX helpers for asynchronous copies ---------------------------------------
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p)
+{
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ uint64_t global_ns()
+{
+    uint64_t t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+// Wait for a plane with a time limit (about one second); on expiry record
+// TL_ETIMEOUT in the lattice status and return false.
+constexpr uint64_t kWaitLimitNs = 1000000000ull;
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, Scalars *sc)
+{
+    if (mbar_test(bar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    for (;;) {
+        for (int i = 0; i < 256; ++i)
+            if (mbar_test(bar, parity)) return true;
+        if (global_ns() - t0 > kWaitLimitNs) {
+            atomicCAS(&sc->status, TL_OK, TL_ETIMEOUT);
+            return false;
+        }
+    }
+}
+
 // ---- variant 1: register streaming with a per-thread prefetch ring -------------
 // Each thread owns its 128-bit words.  The HBM stream (the stored phi and pi
 // of its own sites, plane after plane) is prefetched D planes ahead with
@@ -715,6 +771,206 @@ __device__ __forceinline__ void ldg_tile(const Model &m, const FieldPtrs &fp, co
     reduce_tile<NQ>(acc, accd, flushed, (int)blockDim.x >> 5, red, [] { __syncthreads(); }, m, c, sc, slots, bid, nblocks);
 }
 
+// The same tile for FP64 in CTAs of 256 threads.  There the FP64 pipe is the bound,
+// and of a site's 20 operations in ldg_tile four are drifts: its own and, since
+// every thread drifts what it reads, its neighbours'.  Here a site is drifted
+// once, by its own thread, and its neighbours read it from a plane in shared
+// memory, double-buffered (one barrier a plane); the tile's border is
+// drifted by its first threads (txt x ty = 32 x 8: 144 sites for 512).  Words of
+// plane z + 2 and the border of z + 1 are on their way while z is updated.
+constexpr int kSharedPlane = 704;  // values of (ty + 2) x (2 txt + 4), ty = 256/txt: 680 at txt 8 and 32
+
+template <int NF, bool MEASURE>
+__device__ __forceinline__ void shared_tile(const Model &m, const FieldPtrs &fp, const PassCoef &c, int txt, int ty,
+                                            int zc, int bx, int by, int bz, unsigned bid, unsigned nblocks, Scalars *sc,
+                                            double *slots, uint64_t *ready, uint32_t &parity)
+{
+    using T = double;
+    constexpr int W = 2, NQ = 2 * NF + 1;
+    __shared__ __align__(16) T planes[3][NF][kSharedPlane];
+    __shared__ T coefs[kCoefs];
+    __shared__ double red[256 / 32][NQ];
+    const int N = m.N, tid = threadIdx.x;
+    const int tx = tid % txt, tyi = tid / txt;
+    const int xs = bx * txt * W, ys = by * ty, x0 = xs + tx * W, y = ys + tyi;
+    const int z0 = bz * zc, z1 = min(z0 + zc, N);
+    const bool active = tyi < ty && x0 < N && y < N;
+    const size_t NN = (size_t)m.pplane, P = (size_t)m.pitch;
+    const size_t at = (size_t)y * P + x0;
+    const int pitch = txt * W + 4, own = (tyi + 1) * pitch + 2 + tx * W;
+    // this thread's part of the border: two sites of the rows before and after the
+    // tile (the first 2 txt threads) or one of the columns (the next 2 ty)
+    int border = 0, to = 0;
+    size_t from = 0;
+    {
+        const int xe = min(xs + txt * W, N), ye = min(ys + ty, N);
+        const int h = tid - 2 * txt;
+        if (h < 0) {
+            const bool after = tid >= txt;
+            const int bxx = xs + (after ? tid - txt : tid) * W, yy = after ? (ye == N ? 0 : ye) : (ys == 0 ? N : ys) - 1;
+            border = bxx < N ? 2 : 0;
+            from = (size_t)yy * P + bxx;
+            to = (after ? ye - ys + 1 : 0) * pitch + 2 + bxx - xs;
+        } else if (h < 2 * ty) {
+            const bool after = h >= ty;
+            const int r = after ? h - ty : h, xx = after ? (xe == N ? 0 : xe) : (xs == 0 ? N : xs) - 1;
+            border = ys + r < N ? 1 : 0;
+            from = (size_t)(ys + r) * P + xx;
+            to = (r + 1) * pitch + (after ? 2 + xe - xs : 1);
+        }
+    }
+    const T *phs[NF], *pis[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        phs[f] = static_cast<const T *>(fp.phi_in[f]);
+        pis[f] = static_cast<const T *>(fp.pi_in[f]);
+    }
+    auto plane = [&](int zz) -> size_t { return (size_t)(zz < 0 ? zz + N : zz >= N ? zz - N : zz) * NN; };
+    T zm[NF][W] = {}, cu[NF][W] = {}, pc[NF][W] = {}, rph[NF][W] = {}, rpi[NF][W] = {}, hph[NF][W] = {}, hpi[NF][W] = {};
+    auto load_own = [&](int zz, T (&ph)[NF][W], T (&pi)[NF][W]) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            load_vec(phs[f] + plane(zz) + at, ph[f]);
+            load_vec(pis[f] + plane(zz) + at, pi[f]);
+        }
+    };
+    auto load_border = [&](int zz) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            if (border == 2) {
+                load_vec(phs[f] + plane(zz) + from, hph[f]);
+                load_vec(pis[f] + plane(zz) + from, hpi[f]);
+            } else if (border == 1) {
+                hph[f][0] = __ldg(phs[f] + plane(zz) + from);
+                hpi[f][0] = __ldg(pis[f] + plane(zz) + from);
+            }
+        }
+    };
+    T pm[NF][W] = {};
+    if (active) {
+        load_own(z0 - 1, zm, pm);
+        load_own(z0, cu, pc);
+        load_own(z0 + 1, rph, rpi);
+    }
+    load_border(z0);
+    if (tid < 32) share_coefs(coefs, m, c, sc);
+    __syncthreads();
+    const Coefs<T, NF> k = load_coefs<T, NF>(coefs);
+    bool alive = true;
+    auto put = [&](int b, const T (&v)[NF][W]) {  // this thread's words of a plane and its part of the border
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            if (active) store_vec(&planes[b][f][own], v[f]);
+            if (border) planes[b][f][to] = fma_t(k.drift, hpi[f][0], hph[f][0]);
+            if (border == 2) planes[b][f][to + 1] = fma_t(k.drift, hpi[f][1], hph[f][1]);
+        }
+        __syncwarp();
+        if ((tid & 31) == 0) mbar_arrive(ready);
+    };
+    const bool flushed = z1 - z0 > kFlush;
+    T acc[NQ], accd[NQ];  // summed as in ldg_tile
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) acc[i] = accd[i] = 0.0;
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            zm[f][j] = fma_t(k.drift, pm[f][j], zm[f][j]);
+            cu[f][j] = fma_t(k.drift, pc[f][j], cu[f][j]);
+        }
+    put(0, cu);
+    if (z0 + 1 < z1) load_border(z0 + 1);
+    T *pho[NF], *pio[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        pho[f] = static_cast<T *>(fp.phi_out[f]);
+        pio[f] = static_cast<T *>(fp.pi_out[f]);
+    }
+    int b = 0;  // plane z's place in the ring
+    for (int zf = z0; zf < z1; zf += kFlush) {
+        const int ze = min(zf + kFlush, z1);
+        for (int z = zf; z < ze; ++z) {
+            const int bn = b == 2 ? 0 : b + 1;
+            T zp[NF][W], pnext[NF][W];
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int j = 0; j < W; ++j) {
+                    pnext[f][j] = rpi[f][j];
+                    zp[f][j] = fma_t(k.drift, rpi[f][j], rph[f][j]);
+                }
+            // plane z is in place once every warp has arrived for it; all have then read z - 2, whose place z + 1 takes
+            if (alive) alive = mbar_wait_bounded(ready, parity, sc);
+            parity ^= 1u;
+            if (z + 1 < z1) {
+                put(bn, zp);
+                if (active) load_own(z + 2, rph, rpi);
+                if (z + 2 < z1) load_border(z + 2);
+            }
+            if (active) {
+                T ym[NF][W], yp[NF][W], xl[NF], xr[NF];
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    const T *s = &planes[b][f][own];
+                    load_vec_s(s - pitch, ym[f]);
+                    load_vec_s(s + pitch, yp[f]);
+                    xl[f] = s[-1];
+                    xr[f] = s[W];
+                }
+                T pnew[NF][W];
+                site_update<T, NF, W>(k, cu, zm, zp, ym, yp, xl, xr, pc, pnew, acc);
+                if (!MEASURE) {
+                    const size_t pz = (size_t)z * NN;
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) {
+                        store_vec_cs(pho[f] + pz + at, cu[f]);
+                        store_vec_cs(pio[f] + pz + at, pnew[f]);
+                    }
+                    if (m.ghosts) store_ghosts<T, NF, W>(pho, pio, cu, pnew, pz, x0, y, N, (long long)P);
+                }
+            }
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int j = 0; j < W; ++j) {
+                    zm[f][j] = cu[f][j];
+                    cu[f][j] = zp[f][j];
+                    pc[f][j] = pnext[f][j];
+                }
+            b = bn;
+        }
+        if (flushed) {
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                accd[i] += acc[i];
+                acc[i] = 0.0;
+            }
+        }
+    }
+    reduce_tile<NQ>(acc, accd, flushed, 8, red, [] { __syncthreads(); }, m, c, sc, slots, bid, nblocks);
+}
+
+// Chunks of one or two planes, which are for lattices that do not fill the GPU and
+// wait for latencies, stay with ldg_tile (one field 32^3 9.1 against 9.3 us, 40^3
+// 11.2 against 11.6; from 64^3 on, 4 planes, 20.9 -> 17.7, 128^3 96 -> 82, 256^3 672 ->
+// 553, 512^3 5094 -> 4202), three fields too (their planes leave too little shared
+// memory; two: 100^3 93 -> 87, 256^3 1325 -> 1214).
+template <typename T, int NF>
+constexpr bool kSharedTile = sizeof(T) == 8 && NF <= 2;
+constexpr int kSharedChunk = 3;  // planes, at least
+
+template <int NF, bool MEASURE>
+__global__ void __launch_bounds__(256, 2) fused_pass_shared(Model m, FieldPtrs fp, PassCoef c, int txt, int ty, int zc,
+                                                            Scalars *sc, double *slots)
+{
+    __shared__ uint64_t ready;
+    uint32_t parity = 0;
+    if (threadIdx.x == 0) mbar_init(&ready, 256 / 32);  // a barrier of the tile comes before its first use
+    pass_begin();
+    shared_tile<NF, MEASURE>(m, fp, c, txt, ty, zc, blockIdx.x, blockIdx.y, blockIdx.z, grid_bid(), grid_nblocks(), sc,
+                             slots, &ready, parity);
+}
+
 template <typename T, int NF, bool MEASURE, int D, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) fused_pass_ldg(Model m, FieldPtrs fp, PassCoef c, int txt, int ty, int zc,
                                                             Scalars *sc, double *slots)
@@ -761,6 +1017,9 @@ __global__ void __launch_bounds__(256, 2) fused_pass_group(const BatchJob *__res
         __syncthreads();
     }
     const unsigned *first = staged ? s_first : first_item;
+    [[maybe_unused]] __shared__ uint64_t ready;
+    [[maybe_unused]] uint32_t parity = 0;
+    if (kSharedTile<T, NF> && D == 0 && threadIdx.x == 0) mbar_init(&ready, 256 / 32);
     pass_begin();
     for (unsigned item = blockIdx.x; item < total; item += gridDim.x) {
         int lo = 0, hi = njobs - 1;  // last job whose first item <= item
@@ -774,7 +1033,11 @@ __global__ void __launch_bounds__(256, 2) fused_pass_group(const BatchJob *__res
         const int bx = (int)(local % (unsigned)j.gx);
         const int by = (int)((local / (unsigned)j.gx) % (unsigned)j.gy);
         const int bz = (int)(local / ((unsigned)j.gx * (unsigned)j.gy));
-        ldg_tile<T, NF, false, D>(j.m, j.fp, c, j.txt, j.ty, j.zc, bx, by, bz, local, j.nblocks, j.sc, j.slots, ring);
+        if constexpr (kSharedTile<T, NF> && D == 0)
+            shared_tile<NF, false>(j.m, j.fp, c, j.txt, j.ty, j.zc, bx, by, bz, local, j.nblocks, j.sc, j.slots, &ready,
+                                   parity);
+        else
+            ldg_tile<T, NF, false, D>(j.m, j.fp, c, j.txt, j.ty, j.zc, bx, by, bz, local, j.nblocks, j.sc, j.slots, ring);
         __syncthreads();  // the shared sums and coefficients are the next item's
     }
 }
@@ -804,7 +1067,7 @@ static cudaError_t launch_group_t(int prefetch, const BatchJob *jobs, const unsi
     const int D = prefetch > 0 ? 3 : 0;
     const size_t smem = group_smem_bytes(njobs, NF, D);
     auto kern = D ? fused_pass_group<T, NF, 3> : fused_pass_group<T, NF, 0>;
-    if (smem > 48 * 1024) {
+    if (smem > 12 * 1024) {  // with up to 34 KB that are static it may pass 48 KB
         // the opt-in limit for this kernel (per device, set once; an equal or smaller request needs nothing)
         static std::atomic<size_t> configured[64][2];
         int dev = 0;
@@ -822,58 +1085,6 @@ static cudaError_t launch_group_t(int prefetch, const BatchJob *jobs, const unsi
     }
     return launch_dependent(kern, dim3((unsigned)grid), 256, smem, s, jobs, first_item, njobs, total, c);
 }
-
-// ---- PTX helpers for asynchronous copies ---------------------------------------
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ uint64_t global_ns()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Wait for a plane with a time limit (about one second); on expiry record
-// TL_ETIMEOUT in the lattice status and return false.
-constexpr uint64_t kWaitLimitNs = 1000000000ull;
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, Scalars *sc)
-{
-    if (mbar_test(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    for (;;) {
-        for (int i = 0; i < 256; ++i)
-            if (mbar_test(bar, parity)) return true;
-        if (global_ns() - t0 > kWaitLimitNs) {
-            atomicCAS(&sc->status, TL_OK, TL_ETIMEOUT);
-            return false;
-        }
-    }
-}
-
 
 // ---- variant 2: tiled TMA staging on the ghost-padded layout ---------------------
 // Warps 0..CW-1 compute, warp CW produces.  A CTA owns a tile of txt W x ty
@@ -1592,6 +1803,11 @@ static cudaError_t launch_t(const Model &m, const FieldPtrs &fp, const PassCoef 
         if (big)
             return measure_only ? launch_ldg<T, NF, true, 0, 512>(m, fp, c, g, sc, slots, s)
                                 : launch_ldg<T, NF, false, 0, 512>(m, fp, c, g, sc, slots, s);
+        if constexpr (kSharedTile<T, NF>)
+            if (g.zc >= kSharedChunk) {
+                auto kern = measure_only ? fused_pass_shared<NF, true> : fused_pass_shared<NF, false>;
+                return launch_dependent(kern, g.grid, 256, 0, s, m, fp, c, g.txt, g.ty, g.zc, sc, slots);
+            }
         return measure_only ? launch_ldg<T, NF, true, 0, 256>(m, fp, c, g, sc, slots, s)
                             : launch_ldg<T, NF, false, 0, 256>(m, fp, c, g, sc, slots, s);
     }

@@ -50,6 +50,17 @@ def test_default_shape_equals_plain_streaming(N, nf, dtype):
     same(run(N, nf, dtype, None), run(N, nf, dtype, PLAIN if N >= 16 else dict(kind="stream", z_chunk=N)), dtype)
 
 
+@pytest.mark.parametrize("N,nf,zc,tile_x", [(8, 2, 3, 0), (12, 1, 5, 0), (20, 2, 20, 0), (36, 1, 16, 8), (68, 1, 17, 0),
+                                            (68, 2, 33, 16), (100, 1, 3, 0), (100, 2, 50, 8), (132, 1, 48, 0)])
+def test_shared_planes_equal_plain_streaming(N, nf, zc, tile_x):
+    """FP64 with planes in shared memory (256 threads) against 512 threads, which
+    read their neighbours from memory: tiles cut by both edges of the lattice, rows
+    that straddle warps, chunks around the three planes of the ring and the 16 of
+    a sum, the last one short."""
+    got = run(N, nf, "f64", dict(kind="stream", z_chunk=zc, tile_x=tile_x))
+    same(got, run(N, nf, "f64", dict(kind="stream", z_chunk=min(16, N), threads=512)), "f64")
+
+
 @pytest.mark.parametrize("nf", [1, 2, 3])
 @pytest.mark.parametrize("shape", [dict(kind="tma", warps=7, z_chunk=17), dict(kind="tma", warps=15, z_chunk=40)],
                          ids=["7-17", "15-40"])
@@ -59,15 +70,16 @@ def test_tma_tiles_inside_and_at_the_edge(nf, shape):
     same(run(268, nf, "f32", shape), run(268, nf, "f32", PLAIN), "f32")
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("sizes", [(76, 80, 96), (80, 100, 192), (16, 36)], ids=str)
-def test_batch_members_equal_plain_streaming(sizes):
+def test_batch_members_equal_plain_streaming(sizes, dtype):
     members = [(N, nf) for N in sizes for nf in (1, 2, 3)]
-    lats = [lattice(N, nf, "f32", 7 + i)[0] for i, (N, nf) in enumerate(members)]
+    lats = [lattice(N, nf, dtype, 7 + i)[0] for i, (N, nf) in enumerate(members)]
     with T.Batch(lats) as b:
         b.step(4, 0.01, "verlet")
     for i, (lat, (N, nf)) in enumerate(zip(lats, members)):
         with lat:
-            same((*lat.get_all(), lat.energies().vector()), run(N, nf, "f32", PLAIN, 7 + i), "f32")
+            same((*lat.get_all(), lat.energies().vector()), run(N, nf, dtype, PLAIN, 7 + i), dtype)
 
 
 @pytest.mark.parametrize("alpha", [-1.0, 0.0, 0.5, 1.0, 2.0, 1.0 / 3.0])

@@ -897,6 +897,11 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
     double2 *modes = nullptr;  // N x N x N/2 modes, then (in place) the N^3 field
     if (tl::scratch_alloc((void **)&modes, n3_of(N) * sizeof(double), L->stream) != cudaSuccess)
         return fail(TL_ENOMEM, "scratch allocation for the initial field failed");
+    double *power = nullptr;  // of modes by |n|^2; without it every mode computes its own (below 64^3 a launch costs more)
+    if (N >= 64 && tl::scratch_alloc((void **)&power, tl::mode_powers(N) * sizeof(double), L->stream) != cudaSuccess) {
+        power = nullptr;
+        cudaGetLastError();
+    }
     int rc = TL_OK;
     const bool expanding = L->ex.expanding != 0;
     const double pscale = expanding ? pow(L->ex.a0, 3.0 - L->ex.alpha) : 1.0;
@@ -906,7 +911,7 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
             const bool fluct = which == 0 || spec->fluct_pi;
             void *dst = L->buf[L->cur][which][f];
             if (fluct && spec->A > 0.0) {
-                cudaError_t ce = tl::launch_fill_modes(modes, N, L->kIR, spec->A, spec->meff2[f], which,
+                cudaError_t ce = tl::launch_fill_modes(modes, power, N, L->kIR, spec->A, spec->meff2[f], which,
                                                        spec->fixed_modulus ? 1 : 0, seed, which == 0 ? (uint64_t)f : (uint64_t)(8 + f),
                                                        L->sm_count, L->stream);
                 if (ce != cudaSuccess) { rc = fail(TL_ECUDA, "fill_modes: %s", cudaGetErrorString(ce)); break; }
@@ -923,6 +928,7 @@ int tl_init_fluctuations(tl_lattice *L, uint64_t seed, const tl_init_spec *spec)
         if (rc == TL_OK) rc = used;
     }
     cudaFreeAsync(modes, L->stream);
+    if (power) cudaFreeAsync(power, L->stream);
     if (rc) return rc;
     L->state_mask = (1u << (2 * L->nf)) - 1u;
     L->has_state = true;

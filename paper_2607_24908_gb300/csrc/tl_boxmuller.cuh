@@ -89,6 +89,15 @@ __device__ __forceinline__ void load_box_muller(BoxMullerTable *t)
     __syncthreads();
 }
 
+// (double)k for |k| < 64, by integer instructions (a conversion holds the FP64 pipe).
+__device__ __forceinline__ double small_int(int k)
+{
+    const int a = k < 0 ? -k : k;
+    const int lead = 63 - __clzll((long long)a | 1);  // of 0: 0, with the bit removed below
+    const uint64_t bits = ((uint64_t)(1023 + lead) << 52) + (((uint64_t)(a - (1 << lead))) << (52 - lead));
+    return __longlong_as_double((long long)((a ? bits : 0) | (k < 0 ? 1ull << 63 : 0)));
+}
+
 // -ln(m 2^-53) for an integer 1 <= m <= 2^53.
 __device__ __forceinline__ double neg_log_u53(const BoxMullerTable *t, uint64_t m)
 {
@@ -104,7 +113,7 @@ __device__ __forceinline__ double neg_log_u53(const BoxMullerTable *t, uint64_t 
     q = fma(r, q, -1.0 / 4.0);
     q = fma(r, q, 1.0 / 3.0);
     q = fma(r, q, -1.0 / 2.0);
-    return -fma((double)k, M_LN2, e.y) - fma(r * r, q, r);
+    return -fma(small_int(k), M_LN2, e.y) - fma(r * r, q, r);
 }
 
 // (cos, sin)(2 pi m 2^-53) for an integer 0 <= m < 2^53.

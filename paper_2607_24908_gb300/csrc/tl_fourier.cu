@@ -38,7 +38,20 @@ struct ModeSpec {
 // sqrt(P/L^3) times the Rayleigh factor sqrt(-ln u1), phase 2 pi u2, drawn at
 // the member of each Hermitian pair with the first nonzero of (nx, ny, nz)
 // positive; zero outside 0 < |n| < N/2.
-__device__ __forceinline__ double2 draw_mode(const BoxMullerTable *t, const ModeSpec &p, int nx, int iy, int iz)
+__device__ __forceinline__ double mode_power(const ModeSpec &p, int r2)  // P/L^3, r2 = |n|^2
+{
+    const double om2 = p.kIR2 * (double)r2 + p.m2;
+    return p.amp2 * (p.pi_spectrum ? sqrt(om2) : rsqrt(om2));
+}
+
+__global__ void __launch_bounds__(256) mode_power_kernel(double *power, int count, ModeSpec p)
+{
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < count) power[i] = i ? mode_power(p, i) : 0.0;
+}
+
+__device__ __forceinline__ double2 draw_mode(const BoxMullerTable *t, const double *__restrict__ power, const ModeSpec &p,
+                                             int nx, int iy, int iz)
 {
     const int N = p.N;
     const int ny = signed_mode(iy, N), nz = signed_mode(iz, N);
@@ -48,8 +61,7 @@ __device__ __forceinline__ double2 draw_mode(const BoxMullerTable *t, const Mode
     const int dy = canon ? iy : (iy ? N - iy : 0), dz = canon ? iz : (iz ? N - iz : 0);
     uint64_t w0, w1;
     philox2x64_10(((uint64_t)dz * N + (uint64_t)dy) * N + (uint64_t)nx, p.stream, p.seed, w0, w1);
-    const double om2 = p.kIR2 * (double)r2 + p.m2;
-    const double P = p.amp2 * (p.pi_spectrum ? sqrt(om2) : rsqrt(om2));
+    const double P = power ? __ldg(power + r2) : mode_power(p, r2);
     const double amp = sqrt(p.fixed_modulus ? P : P * neg_log_u53(t, (w0 >> 11) + 1));
     double s, c;
     unit_circle_u53(t, w1 >> 11, c, s);
@@ -64,8 +76,10 @@ __device__ __forceinline__ double2 draw_mode(const BoxMullerTable *t, const Mode
 //
 // Bound by the FP64 pipe: one square root of the whole modulus squared instead
 // of four roots and two divisions, 256^3 1305 -> 996 us a field, and the table
-// form of the logarithm and the circle (tl_boxmuller.cuh), 996 -> 610 us.
-__global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, ModeSpec p)
+// form of the logarithm and the circle (tl_boxmuller.cuh), 996 -> 610 us; P by |n|^2
+// from a table that a small kernel fills first (a root and three operations a mode
+// less, the same values) and integer-to-FP64 conversions by bits, 604 -> 512 us.
+__global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, const double *__restrict__ power, ModeSpec p)
 {
     extern __shared__ double2 root[];
     __shared__ BoxMullerTable table;
@@ -77,12 +91,12 @@ __global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, ModeSpe
         const unsigned row = i / q, k = i - row * q;
         const int iz = row / N, iy = row - (unsigned)iz * N;
         const int my = iy ? N - iy : 0, mz = iz ? N - iz : 0;
-        const double2 a = draw_mode(&table, p, k, iy, iz);
+        const double2 a = draw_mode(&table, power, p, k, iy, iz);
         if (k == 0) {  // (1 + i) F1
             modes[(size_t)row * h] = make_double2(a.x - a.y, a.x + a.y);
             continue;
         }
-        const double2 b = draw_mode(&table, p, h - k, my, mz);
+        const double2 b = draw_mode(&table, power, p, h - k, my, mz);
         const double2 w = root[k];
         const double dx = a.x - b.x, dy = a.y + b.y;
         const double zx = -(w.x * dy + w.y * dx), zy = w.x * dx - w.y * dy;
@@ -96,7 +110,7 @@ __global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, ModeSpe
 // layouts' FP32 form and N is a multiple of 4): 16- and 32-byte accesses, one
 // index decomposition for the four.  Conversions are integer instructions
 // (tl_bits.cuh; a field without fluctuations is converted once, on the host): us,
-// 256^3 FP32, with F2F -> without: assemble 70, fill 69 -> 12.
+// 256^3 FP32, with F2F -> without: fill 69 -> 18.
 template <typename T>
 struct Four;
 template <>
@@ -297,13 +311,19 @@ static unsigned grid_for(size_t n, int sm_count, int per_sm)
     return (unsigned)(g < cap ? g : cap);
 }
 
-cudaError_t launch_fill_modes(double2 *modes, int N, double kIR, double A, double m2, int pi_spectrum,
+cudaError_t launch_fill_modes(double2 *modes, double *power, int N, double kIR, double A, double m2, int pi_spectrum,
                               int fixed_modulus, uint64_t seed, uint64_t stream, int sm_count, cudaStream_t s)
 {
     const double L = 2.0 * M_PI / kIR;
     const ModeSpec p{N, kIR * kIR, m2, A / (2.0 * L * L * L), pi_spectrum, fixed_modulus, seed, stream};
     const size_t total = (size_t)N * N * (N / 4 + 1);
-    fill_modes_kernel<<<grid_for(total, sm_count, 8), 256, (N / 4 + 1) * sizeof(double2), s>>>(modes, p);
+    if (power) {
+        const int count = mode_powers(N);
+        mode_power_kernel<<<(count + 255) / 256, 256, 0, s>>>(power, count, p);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    fill_modes_kernel<<<grid_for(total, sm_count, 8), 256, (N / 4 + 1) * sizeof(double2), s>>>(modes, power, p);
     return cudaGetLastError();
 }
 

@@ -18,8 +18,10 @@ namespace tl {
 // thirds of the time of a real-to-complex transform (256^3: 1.45 against
 // 2.27 ms, 192^3 0.65 against 0.93; sizes with large prime factors 5-10%).
 
-// The modes C of a Gaussian random field (see tl_init_spec), for the inverse transform.
-cudaError_t launch_fill_modes(double2 *modes, int N, double kIR, double A, double m2, int pi_spectrum,
+// The modes C of a Gaussian random field (see tl_init_spec), for the inverse
+// transform.  power: scratch for mode_powers(N) values, or NULL.
+constexpr int mode_powers(int N) { return N * N / 4; }
+cudaError_t launch_fill_modes(double2 *modes, double *power, int N, double kIR, double A, double m2, int pi_spectrum,
                               int fixed_modulus, uint64_t seed, uint64_t stream, int sm_count, cudaStream_t s);
 // The padded array at dst = base + scale * delta (delta dense; may be NULL), ghost rows included.
 cudaError_t launch_assemble(int dtype, void *dst, const double *delta, double base, double scale, int N, long long P,

@@ -35,10 +35,8 @@ __global__ void set_background_kernel(Model m, Scalars *sc, double a, double b) 
 // for 16 clocks whatever its lanes do, so that a pass takes as long as the SM
 // with the most warp-planes: per warp and plane about 50 instructions a field (57
 // in chunks of one plane, which drift three planes for one), and per CTA its
-// sums and latencies, about 60.  Measured against this estimate (us, one field,
-// one plane a chunk -> chosen): 64^3 35.7 -> 20.8 (3 planes; 4: 19.7), 96^3 81.5 ->
-// 49 (14 planes), 128^3 96 (7 planes; 32: 101), 140^3 127 (20 planes; 32: 197), 212^3
-// 428 (20; 32: 447).  32^3 takes tiles of 16 x 8 threads on 128 SMs, not 16 x 16 on 64.
+// sums and latencies, about 60.  That estimate gives the rows of thin tiles: 32^3 takes
+// tiles of 16 x 8 threads on 128 SMs, not 16 x 16 on 64.
 
 constexpr int kThinChunk = 3;  // chunks up to here may have tiles of fewer rows
 
@@ -61,13 +59,13 @@ static int f64_tile_rows(int N, int gx, int txt, int ty_max, int zc, int sms)
     return best;
 }
 
-// FP64 chunk with one or two fields (shared_tile): the cheapest by (waves of two
+// FP64 chunk (shared_tile): the cheapest by (waves of two
 // CTAs per SM) x (warps per CTA x planes), where a last wave of at most one CTA per
 // SM counts 0.6 and a CTA no less than 6 warps.  Over 36 lattices of 32^3 to 384^3 the
 // choice is 0.6% slower than the best of a sweep (8% at 144^3 with two fields), that
-// of the estimate above, made for ldg_tile, 5% (us: 144^3 155 -> 127, 160^3 199 -> 160,
-// 212^3 396 -> 355, 300^3 1090 -> 932).  Two fields keep 32 planes from 128^3 unless
-// another is estimated 4% cheaper (256^3 1216, 37 planes 1200).
+// of the estimate above 5% (us: 144^3 155 -> 127, 160^3 199 -> 160, 212^3 396 -> 355, 300^3
+// 1090 -> 932; three fields 160^3 636 -> 501).  Two fields keep 32 planes from 128^3
+// unless another is estimated 4% cheaper (256^3 1216, 37 planes 1200).
 static double f64_shared_cost(int N, int gx, int txt, int ty, int zc, int sms)
 {
     const long ctas = (long)gx * ((N + ty - 1) / ty) * ((N + zc - 1) / zc), last = ctas % (2 * sms);
@@ -77,16 +75,13 @@ static double f64_shared_cost(int N, int gx, int txt, int ty, int zc, int sms)
     return waves * (warps * (zc + 0.3) + 3.0);
 }
 
-// FP64 chunk: the cheapest; with three fields from 128^3 32 planes and from 512^3
-// 64 (the best of a measured sweep) unless another is estimated 5% cheaper.
 static int f64_chunk(int N, int nf, int gx, int txt, int ty_max, int sms)
 {
     auto cost = [&](int zc) {
-        const int ty = f64_tile_rows(N, gx, txt, ty_max, zc, sms);
-        return nf <= 2 ? f64_shared_cost(N, gx, txt, ty, zc, sms) : f64_cost(N, gx, txt, ty, zc, sms);
+        return f64_shared_cost(N, gx, txt, f64_tile_rows(N, gx, txt, ty_max, zc, sms), zc, sms);
     };
-    int best = nf == 3 && N >= 512 ? 64 : N >= 128 ? 32 : 1;
-    double least = cost(best) * (N < 128 || nf == 1 ? 1.0 : nf == 2 ? 0.96 : 0.95);
+    int best = N >= 128 ? 32 : 1;
+    double least = cost(best) * (N >= 128 && nf == 2 ? 0.96 : 1.0);
     for (int zc = 1; zc <= N && zc <= 128; ++zc)
         if (cost(zc) < least) least = cost(zc), best = zc;
     return best;

@@ -783,11 +783,11 @@ constexpr int kSharedPlane = 704;  // values of (ty + 2) x (2 txt + 4), ty = 256
 template <int NF, bool MEASURE>
 __device__ __forceinline__ void shared_tile(const Model &m, const FieldPtrs &fp, const PassCoef &c, int txt, int ty,
                                             int zc, int bx, int by, int bz, unsigned bid, unsigned nblocks, Scalars *sc,
-                                            double *slots, uint64_t *ready, uint32_t &parity)
+                                            double *slots, double *ring, uint64_t *ready, uint32_t &parity)
 {
     using T = double;
     constexpr int W = 2, NQ = 2 * NF + 1;
-    __shared__ __align__(16) T planes[3][NF][kSharedPlane];
+    T(*planes)[NF][kSharedPlane] = reinterpret_cast<T(*)[NF][kSharedPlane]>(ring);  // three planes
     __shared__ T coefs[kCoefs];
     __shared__ double red[256 / 32][NQ];
     const int N = m.N, tid = threadIdx.x;
@@ -950,25 +950,30 @@ __device__ __forceinline__ void shared_tile(const Model &m, const FieldPtrs &fp,
     reduce_tile<NQ>(acc, accd, flushed, 8, red, [] { __syncthreads(); }, m, c, sc, slots, bid, nblocks);
 }
 
-// Chunks of one or two planes, which are for lattices that do not fill the GPU and
-// wait for latencies, stay with ldg_tile (one field 32^3 9.1 against 9.3 us, 40^3
-// 11.2 against 11.6; from 64^3 on, 4 planes, 20.9 -> 17.7, 128^3 96 -> 82, 256^3 672 ->
-// 553, 512^3 5094 -> 4202), three fields too (their planes leave too little shared
-// memory; two: 100^3 93 -> 87, 256^3 1325 -> 1214).
-template <typename T, int NF>
-constexpr bool kSharedTile = sizeof(T) == 8 && NF <= 2;
-constexpr int kSharedChunk = 3;  // planes, at least
+// Chunks of one or two planes (three fields: three), which are for lattices that do
+// not fill the GPU and wait for latencies, stay with ldg_tile (one field 32^3 9.1
+// against 9.3 us, 40^3 11.2 against 11.6, three 56^3 32.5 against 33.2).  From there on
+// (us, ldg_tile -> here, chunks by f64_chunk): one field 64^3 20.9 -> 17.7, 128^3 96 -> 82,
+// 256^3 672 -> 553, 512^3 5094 -> 4202; two 100^3 93 -> 87, 256^3 1325 -> 1214; three, whose
+// registers spill, 128^3 257 -> 249, 256^3 1913 -> 1780.  A batch takes it for one and
+// two fields (32 jobs 15.1 -> 13.8 ms a call).
+template <int NF>
+constexpr int kSharedChunk = NF == 3 ? 4 : 3;  // planes, at least
 
+template <typename T, int NF>
+constexpr bool kSharedGroup = sizeof(T) == 8 && NF <= 2;
+constexpr size_t shared_planes_bytes(int nf) { return (size_t)3 * nf * kSharedPlane * sizeof(double); }
 template <int NF, bool MEASURE>
 __global__ void __launch_bounds__(256, 2) fused_pass_shared(Model m, FieldPtrs fp, PassCoef c, int txt, int ty, int zc,
                                                             Scalars *sc, double *slots)
 {
+    extern __shared__ __align__(16) unsigned char ring_raw[];
     __shared__ uint64_t ready;
     uint32_t parity = 0;
     if (threadIdx.x == 0) mbar_init(&ready, 256 / 32);  // a barrier of the tile comes before its first use
     pass_begin();
     shared_tile<NF, MEASURE>(m, fp, c, txt, ty, zc, blockIdx.x, blockIdx.y, blockIdx.z, grid_bid(), grid_nblocks(), sc,
-                             slots, &ready, parity);
+                             slots, reinterpret_cast<double *>(ring_raw), &ready, parity);
 }
 
 template <typename T, int NF, bool MEASURE, int D, int NT>
@@ -1017,9 +1022,10 @@ __global__ void __launch_bounds__(256, 2) fused_pass_group(const BatchJob *__res
         __syncthreads();
     }
     const unsigned *first = staged ? s_first : first_item;
+    [[maybe_unused]] __shared__ __align__(16) double planes[kSharedGroup<T, NF> && D == 0 ? 3 * NF * kSharedPlane : 2];
     [[maybe_unused]] __shared__ uint64_t ready;
     [[maybe_unused]] uint32_t parity = 0;
-    if (kSharedTile<T, NF> && D == 0 && threadIdx.x == 0) mbar_init(&ready, 256 / 32);
+    if (kSharedGroup<T, NF> && D == 0 && threadIdx.x == 0) mbar_init(&ready, 256 / 32);
     pass_begin();
     for (unsigned item = blockIdx.x; item < total; item += gridDim.x) {
         int lo = 0, hi = njobs - 1;  // last job whose first item <= item
@@ -1033,9 +1039,9 @@ __global__ void __launch_bounds__(256, 2) fused_pass_group(const BatchJob *__res
         const int bx = (int)(local % (unsigned)j.gx);
         const int by = (int)((local / (unsigned)j.gx) % (unsigned)j.gy);
         const int bz = (int)(local / ((unsigned)j.gx * (unsigned)j.gy));
-        if constexpr (kSharedTile<T, NF> && D == 0)
-            shared_tile<NF, false>(j.m, j.fp, c, j.txt, j.ty, j.zc, bx, by, bz, local, j.nblocks, j.sc, j.slots, &ready,
-                                   parity);
+        if constexpr (kSharedGroup<T, NF> && D == 0)
+            shared_tile<NF, false>(j.m, j.fp, c, j.txt, j.ty, j.zc, bx, by, bz, local, j.nblocks, j.sc, j.slots,
+                                   planes, &ready, parity);
         else
             ldg_tile<T, NF, false, D>(j.m, j.fp, c, j.txt, j.ty, j.zc, bx, by, bz, local, j.nblocks, j.sc, j.slots, ring);
         __syncthreads();  // the shared sums and coefficients are the next item's
@@ -1778,6 +1784,18 @@ static cudaError_t launch_tma_group_t(int stages, size_t smem, const BatchJob *j
     return launch_dependent(kern, dim3(total), 256, smem, s, jobs, first_item, njobs, c, stages);
 }
 
+template <int NF, bool MEASURE>
+static cudaError_t launch_shared(const Model &m, const FieldPtrs &fp, const PassCoef &c, const PassGeom &g, Scalars *sc,
+                                 double *slots, cudaStream_t s)
+{
+    static std::atomic<size_t> configured[kMaxDevices][2];
+    auto kern = fused_pass_shared<NF, MEASURE>;
+    constexpr size_t smem = shared_planes_bytes(NF);
+    cudaError_t e = ensure_smem_attribute(kern, smem, configured, 0);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(kern, g.grid, 256, smem, s, m, fp, c, g.txt, g.ty, g.zc, sc, slots);
+}
+
 template <typename T, int NF, bool MEASURE, int D, int NT>
 static cudaError_t launch_ldg(const Model &m, const FieldPtrs &fp, const PassCoef &c, const PassGeom &g, Scalars *sc,
                               double *slots, cudaStream_t s)
@@ -1803,11 +1821,10 @@ static cudaError_t launch_t(const Model &m, const FieldPtrs &fp, const PassCoef 
         if (big)
             return measure_only ? launch_ldg<T, NF, true, 0, 512>(m, fp, c, g, sc, slots, s)
                                 : launch_ldg<T, NF, false, 0, 512>(m, fp, c, g, sc, slots, s);
-        if constexpr (kSharedTile<T, NF>)
-            if (g.zc >= kSharedChunk) {
-                auto kern = measure_only ? fused_pass_shared<NF, true> : fused_pass_shared<NF, false>;
-                return launch_dependent(kern, g.grid, 256, 0, s, m, fp, c, g.txt, g.ty, g.zc, sc, slots);
-            }
+        if constexpr (sizeof(T) == 8)
+            if (g.zc >= kSharedChunk<NF>)
+                return measure_only ? launch_shared<NF, true>(m, fp, c, g, sc, slots, s)
+                                    : launch_shared<NF, false>(m, fp, c, g, sc, slots, s);
         return measure_only ? launch_ldg<T, NF, true, 0, 256>(m, fp, c, g, sc, slots, s)
                             : launch_ldg<T, NF, false, 0, 256>(m, fp, c, g, sc, slots, s);
     }

@@ -51,7 +51,8 @@ def test_default_shape_equals_plain_streaming(N, nf, dtype):
 
 
 @pytest.mark.parametrize("N,nf,zc,tile_x", [(8, 2, 3, 0), (12, 1, 5, 0), (20, 2, 20, 0), (36, 1, 16, 8), (68, 1, 17, 0),
-                                            (68, 2, 33, 16), (100, 1, 3, 0), (100, 2, 50, 8), (132, 1, 48, 0)])
+                                            (68, 2, 33, 16), (100, 1, 3, 0), (100, 2, 50, 8), (132, 1, 48, 0), (20, 3, 4, 0),
+                                            (76, 3, 34, 0)])
 def test_shared_planes_equal_plain_streaming(N, nf, zc, tile_x):
     """FP64 with planes in shared memory (256 threads) against 512 threads, which
     read their neighbours from memory: tiles cut by both edges of the lattice, rows

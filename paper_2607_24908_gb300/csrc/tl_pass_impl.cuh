@@ -1392,7 +1392,7 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
 // producer makes them visible to the tensor-map proxy before their first use.
 // Every compute warp takes part in every tile's ring traffic (a warp without
 // sites only waits and releases), so the "empty" barriers count all of them.
-template <typename T, int NF, bool MEASURE, bool GLOBAL_MAPS = false>
+template <typename T, int NF, bool MEASURE>
 __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, const PassCoef &c, int txt, int ty,
                                           int zc, int S, int lpad, const TmaMaps *maps, Scalars *sc, double *slots,
                                           unsigned first, unsigned stride, unsigned nitems, int gx, int gy)
@@ -1433,14 +1433,6 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
     pass_begin();
     if (producer) {
         if (lane == 0) {
-            if constexpr (GLOBAL_MAPS) {
-#pragma unroll
-                for (int kk = 0; kk < 3; ++kk)
-#pragma unroll
-                    for (int i = 0; i < 2 * NF; ++i)
-                        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&maps->map[kk][i])
-                                     : "memory");
-            }
             // plane count g and its ring stage ps and phase pph, advanced
             // incrementally (no division in the loop)
             unsigned g = 0, issued = 0, pph = 0;
@@ -1671,8 +1663,9 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
 // 512^3 0.069 / 0.205 / 0.418 ms in tma_tile against 0.103 / 0.322 / 0.673;
 // two fields 256^3, 640^3 and 1024^3 0.106, 1.329 and 5.397 ms in tma_items
 // against 0.111, 1.332 and 5.453, 320^3, 384^3 and 512^3 0.219, 0.309 and
-// 0.691 in tma_tile against 0.244, 0.325 and 0.705; three fields spill less
-// in tma_tile.
+// 0.691 in tma_tile against 0.244, 0.325 and 0.705, 192^3 0.064 against 0.072 (196^3
+// and 200^3 0.061 in tma_items against 0.064); three fields spill less in tma_tile.
+// A batch takes tma_tile (96 jobs of 32^3 ... 128^3 18.34 -> 17.96 ms a call).
 template <typename T, int NF, bool MEASURE, bool ITEMS, bool GLOBAL_MAPS = false>
 __device__ __forceinline__ void tma_one_tile(const Model &m, const FieldPtrs &fp, const PassCoef &c, int txt, int ty,
                                              int zc, int S, int lpad, const TmaMaps *maps, Scalars *sc, double *slots,
@@ -1683,13 +1676,13 @@ __device__ __forceinline__ void tma_one_tile(const Model &m, const FieldPtrs &fp
         const int bz = (int)(item / ((unsigned)gx * (unsigned)gy));
         tma_tile<T, NF, MEASURE, GLOBAL_MAPS>(m, fp, c, txt, ty, zc, S, lpad, maps, sc, slots, bx, by, bz, item, nitems);
     } else {
-        tma_items<T, NF, MEASURE, GLOBAL_MAPS>(m, fp, c, txt, ty, zc, S, lpad, maps, sc, slots, item, nitems, nitems, gx,
-                                               gy);
+        static_assert(!GLOBAL_MAPS, "a batch takes tma_tile");
+        tma_items<T, NF, MEASURE>(m, fp, c, txt, ty, zc, S, lpad, maps, sc, slots, item, nitems, nitems, gx, gy);
     }
 }
 
 // The code form a lattice's TMA pass takes (see tma_one_tile).
-__host__ __device__ constexpr bool tma_items_form(int nf, int N) { return nf == 2 && (N <= 256 || N >= 640); }
+__host__ __device__ constexpr bool tma_items_form(int nf, int N) { return nf == 2 && ((N > 192 && N <= 256) || N >= 640); }
 
 template <typename T, int NF, bool MEASURE, int NTHR, bool ITEMS>
 __global__ void __launch_bounds__(NTHR, (NTHR <= 256 ? 2 : 1)) fused_pass_tma(Model m, FieldPtrs fp, PassCoef c, int txt, int ty, int zc,
@@ -1724,7 +1717,7 @@ __global__ void __launch_bounds__(256, 2) fused_pass_tma_group(const BatchJob *_
     const unsigned local = blockIdx.x - __ldg(first_item + s_job);
     // two fields in the multi-tile code form, as for the small lattices batches
     // hold (either form gives the same numbers)
-    tma_one_tile<T, NF, false, NF == 2, true>(j.m, j.fp, c, j.txt, j.ty, j.zc, S, j.lpad, j.maps, j.sc, j.slots, local,
+    tma_one_tile<T, NF, false, false, true>(j.m, j.fp, c, j.txt, j.ty, j.zc, S, j.lpad, j.maps, j.sc, j.slots, local,
                                               j.nblocks, j.gx, j.gy);
 }
 

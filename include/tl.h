@@ -162,10 +162,10 @@ int tl_set_potential(tl_lattice *lat, const tl_potential *pot);
  * Sec. 3.5); the spectrum A/(2 omega_k) is the workloads' vacuum spectrum.
  * Draw the initial state (see tl_init_spec), set a = a0 and, when expanding,
  * b = a0^(1+alpha) sqrt(mu2 rho0/3) with rho0 the lattice-averaged K+G+V of
- * that state.  Uses cuFFT (complex, FP64) and temporary device memory of about
- * 8 N^3 bytes, from a pool of the library's that keeps up to 1 GiB of it (and
- * of tl_spectrum's) per device between calls, until the device's last lattice
- * is destroyed.  Resets step and time to 0. */
+ * that state.  Transforms in FP64 (cuFFT for N other than 2^m, 3 2^m and 5 2^m
+ * from 64 to 1024); takes temporary device memory of about 8 N^3 bytes, from a
+ * pool of the library's that keeps up to 1 GiB of it (and of tl_spectrum's) per
+ * device between calls, until the device's last lattice is destroyed.  Resets step and time to 0. */
 int tl_init_fluctuations(tl_lattice *lat, uint64_t seed, const tl_init_spec *spec);
 
 /* Passage: Sec. 4, the kick-drift leapfrog of the phi^4 benchmark (kick
@@ -469,9 +469,8 @@ int tl_autotune(tl_lattice *lat, double *best_ms_per_pass);
  * when it is FP32 and N >= 192 (compute warps and z-chunk chosen from N, the
  * field count and the SM count, to run in few full waves of CTAs, up to N = 495;
  * 15 compute warps and measured z-chunks from there), on
- * TL_PASS_STREAM otherwise (where those measured faster; z-chunks chosen from N
- * and the SM count, FP64 mostly 32 planes from N = 128 and 64 from N = 512); the environment
- * variable TL_PASS_VARIANT=tma|ldg overrides that default at creation. */
+ * TL_PASS_STREAM otherwise (where those measured faster; z-chunks chosen from N,
+ * the field count and the SM count); the environment variable TL_PASS_VARIANT=tma|ldg overrides that default at creation. */
 int tl_set_pass_config(tl_lattice *lat, const tl_pass_config *cfg);
 
 /* The launch shape lat runs now, with automatic values resolved. */

@@ -7,7 +7,9 @@
 // is the number of FP64 instructions:
 //  * a butterfly a +- w b with w = c (1 + i t) (or -i c (1 + i t), whichever has
 //    |t| <= 1) takes six fused multiply-adds, two for (1 + i t) b and four for
-//    a +- c (...), instead of eight; the plain ones (w = 1, -i) take four;
+//    a +- c (...), instead of eight (E. Linzer, E. Feig, "Implementation of efficient
+//    FFT algorithms on fused multiply-add architectures", IEEE Trans. Signal
+//    Processing 41, 1993); the plain ones (w = 1, -i) take four;
 //  * roots come from a table, index work, selects, signs and the exchange through
 //    shared memory are other pipes' work and next to free;
 //  * FP32 fields are widened by integer instructions (tl_bits.cuh) as they are

@@ -15,7 +15,8 @@
 // Layout and traffic: each thread owns W = 16/sizeof(T) consecutive x-sites
 // (one 128-bit word per array) of one y-row and marches a chunk of z-planes,
 // keeping phi at z-1, z, z+1 in registers; the neighbour rows and edge sites
-// come through L1/L2 (fused_pass_ldg).  HBM sees each array read once and
+// come through L1/L2 (fused_pass_ldg), from drifted planes in shared memory (FP64,
+// fused_pass_shared) or from tiles that tensor copies stage (fused_pass_tma).  HBM sees each array read once and
 // written once per pass: 4 sizeof(T) bytes per site per field.
 #pragma once
 #include <cuda.h>

@@ -54,7 +54,8 @@ constexpr double sin_turn(int j)
     return x * sum;
 }
 
-struct RawTable {
+// alignas: load_box_muller reads it in 16-byte words.
+struct alignas(16) RawTable {
     double log[kLogEntries][2] = {};
     double circle[kCircleEntries][2] = {};
     constexpr RawTable()
@@ -78,6 +79,8 @@ struct RawTable {
 
 }  // namespace detail
 
+static_assert(alignof(detail::RawTable) >= alignof(double2) && sizeof(detail::RawTable) == sizeof(BoxMullerTable),
+              "the raw table is copied as double2");
 static __device__ const detail::RawTable g_box_muller{};
 
 // Copies the table into a CTA's shared memory (ends with a barrier).

@@ -43,14 +43,17 @@ struct Vec<double> {
     typedef double2 type;
 };
 
+// Field arrays (and shared memory) are read by ordinary loads: a pass may be
+// resident while the pass that writes them runs (pass_begin), and the read-only
+// path (__ldg) wants memory that nothing writes in the kernel's whole lifetime.
 __device__ __forceinline__ void load_vec(const float *p, float (&o)[4])
 {
-    float4 t = __ldg(reinterpret_cast<const float4 *>(p));
+    float4 t = *reinterpret_cast<const float4 *>(p);
     o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
 }
 __device__ __forceinline__ void load_vec(const double *p, double (&o)[2])
 {
-    double2 t = __ldg(reinterpret_cast<const double2 *>(p));
+    double2 t = *reinterpret_cast<const double2 *>(p);
     o[0] = t.x; o[1] = t.y;
 }
 __device__ __forceinline__ void store_vec(float *p, const float (&v)[4])
@@ -60,16 +63,6 @@ __device__ __forceinline__ void store_vec(float *p, const float (&v)[4])
 __device__ __forceinline__ void store_vec(double *p, const double (&v)[2])
 {
     *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
-}
-__device__ __forceinline__ void load_vec_s(const float *p, float (&o)[4])
-{
-    float4 t = *reinterpret_cast<const float4 *>(p);
-    o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
-}
-__device__ __forceinline__ void load_vec_s(const double *p, double (&o)[2])
-{
-    double2 t = *reinterpret_cast<const double2 *>(p);
-    o[0] = t.x; o[1] = t.y;
 }
 // streaming (evict-first) stores: the outputs are read again only by the next pass
 __device__ __forceinline__ void store_vec_cs(float *p, const float (&v)[4])
@@ -682,7 +675,7 @@ __device__ __forceinline__ void ldg_tile(const Model &m, const FieldPtrs &fp, co
             for (int j = 0; j < W; ++j) o[j] = fma_t(k.drift, b[j], a[j]);
         };
         auto cur_one = [&](int f, size_t off) -> T {
-            return fma_t(k.drift, __ldg(pis[f] + off), __ldg(phs[f] + off));
+            return fma_t(k.drift, pis[f][off], phs[f][off]);
         };
         auto plane_off = [&](int zz) -> size_t { return (size_t)(zz >= N ? zz - N : zz) * NN + row + x0; };
         // prefetch this thread's words of plane zz (<= z1) into ring slot d
@@ -711,8 +704,8 @@ __device__ __forceinline__ void ldg_tile(const Model &m, const FieldPtrs &fp, co
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     T a[W];
-                    load_vec_s(slot(d, f, 0), a);
-                    load_vec_s(slot(d, f, 1), pnext[f]);
+                    load_vec(slot(d, f, 0), a);
+                    load_vec(slot(d, f, 1), pnext[f]);
 #pragma unroll
                     for (int j = 0; j < W; ++j) zp[f][j] = fma_t(k.drift, pnext[f][j], a[j]);
                 }
@@ -842,8 +835,8 @@ __device__ __forceinline__ void shared_tile(const Model &m, const FieldPtrs &fp,
                 load_vec(phs[f] + plane(zz) + from, hph[f]);
                 load_vec(pis[f] + plane(zz) + from, hpi[f]);
             } else if (border == 1) {
-                hph[f][0] = __ldg(phs[f] + plane(zz) + from);
-                hpi[f][0] = __ldg(pis[f] + plane(zz) + from);
+                hph[f][0] = phs[f][plane(zz) + from];
+                hpi[f][0] = pis[f][plane(zz) + from];
             }
         }
     };
@@ -913,8 +906,8 @@ __device__ __forceinline__ void shared_tile(const Model &m, const FieldPtrs &fp,
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const T *s = &planes[b][f][own];
-                    load_vec_s(s - pitch, ym[f]);
-                    load_vec_s(s + pitch, yp[f]);
+                    load_vec(s - pitch, ym[f]);
+                    load_vec(s + pitch, yp[f]);
                     xl[f] = s[-1];
                     xr[f] = s[W];
                 }
@@ -1275,8 +1268,8 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
                 T a[W];
-                load_vec_s(arr(s, f, 0) + ctr, a);
-                load_vec_s(arr(s, f, 1) + ctr, pp[f]);
+                load_vec(arr(s, f, 0) + ctr, a);
+                load_vec(arr(s, f, 1) + ctr, pp[f]);
 #pragma unroll
                 for (int j = 0; j < W; ++j) ph[f][j] = fma_t(k.drift, pp[f][j], a[j]);
             }
@@ -1326,14 +1319,14 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const T *ph = arr(s0, f, 0), *pp = arr(s0, f, 1);
-                    if constexpr (kReread) load_vec_s(pp + ctr, pc[f]);
+                    if constexpr (kReread) load_vec(pp + ctr, pc[f]);
                     T a[W], b[W];
-                    load_vec_s(ph + ctr - rowe, a);
-                    load_vec_s(pp + ctr - rowe, b);
+                    load_vec(ph + ctr - rowe, a);
+                    load_vec(pp + ctr - rowe, b);
 #pragma unroll
                     for (int j = 0; j < W; ++j) ym[f][j] = fma_t(k.drift, b[j], a[j]);
-                    load_vec_s(ph + ctr + rowe, a);
-                    load_vec_s(pp + ctr + rowe, b);
+                    load_vec(ph + ctr + rowe, a);
+                    load_vec(pp + ctr + rowe, b);
 #pragma unroll
                     for (int j = 0; j < W; ++j) yp[f][j] = fma_t(k.drift, b[j], a[j]);
                     const T l = __shfl_sync(amask, cu[f][W - 1], src_l);
@@ -1561,8 +1554,8 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     T a[W];
-                    load_vec_s(arr(s, f, 0) + ctr, a);
-                    load_vec_s(arr(s, f, 1) + ctr, pp[f]);
+                    load_vec(arr(s, f, 0) + ctr, a);
+                    load_vec(arr(s, f, 1) + ctr, pp[f]);
 #pragma unroll
                     for (int j = 0; j < W; ++j) ph[f][j] = fma_t(k.drift, pp[f][j], a[j]);
                 }
@@ -1593,12 +1586,12 @@ __device__ __forceinline__ void tma_items(const Model &m, const FieldPtrs &fp, c
                     for (int f = 0; f < NF; ++f) {
                         const T *ph = arr(s0, f, 0), *pp = arr(s0, f, 1);
                         T a[W], b[W];
-                        load_vec_s(ph + ctr - rowe, a);
-                        load_vec_s(pp + ctr - rowe, b);
+                        load_vec(ph + ctr - rowe, a);
+                        load_vec(pp + ctr - rowe, b);
 #pragma unroll
                         for (int j = 0; j < W; ++j) ym[f][j] = fma_t(k.drift, b[j], a[j]);
-                        load_vec_s(ph + ctr + rowe, a);
-                        load_vec_s(pp + ctr + rowe, b);
+                        load_vec(ph + ctr + rowe, a);
+                        load_vec(pp + ctr + rowe, b);
 #pragma unroll
                         for (int j = 0; j < W; ++j) yp[f][j] = fma_t(k.drift, b[j], a[j]);
                         const T l = __shfl_sync(amask, cu[f][W - 1], src_l);

@@ -204,6 +204,7 @@ __device__ __forceinline__ void finish_tile(double sum, const Model &m, const Pa
         __threadfence();
         ticket = atomicAdd(&sc->ticket, 1u);
     }
+    __syncwarp();  // orders the other lanes' reads below after lane 0's ticket (a shuffle orders no memory)
     if (__shfl_sync(0xffffffffu, ticket, 0) != nblocks - 1) return;
     __threadfence();
     const PassEnd was{sc->a, sc->b, sc->wk, sc->wg, sc->pf, sc->ph, sc->ia, sc->time, sc->pending_dt, sc->status};

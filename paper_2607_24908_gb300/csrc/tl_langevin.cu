@@ -129,10 +129,12 @@ __global__ void __launch_bounds__(256) langevin_pass(const T *__restrict__ in, T
     const int y = blockIdx.y * ty + tyi;
     const int z0 = blockIdx.z * zc;
     const int z1 = min(z0 + zc, N);
-    if (!(tyi < ty && x0 < N && y < N)) return;
+    const bool active = tyi < ty && x0 < N && y < N;
     // the x-neighbours are in the adjacent lanes' words; a thread at a row end,
-    // a tile edge or a warp edge loads its own
-    const unsigned lanes = __activemask();
+    // a tile edge or a warp edge loads its own.  The mask of the shuffles is formed
+    // while the warp is whole: every lane that stays is in it
+    const unsigned lanes = __ballot_sync(0xffffffffu, active);
+    if (!active) return;
     const int lane = threadIdx.x & 31;
     const bool own_l = tx == 0 || lane == 0, own_r = tx == txt - 1 || x0 + W == N || lane == 31;
     const int src_l = own_l ? lane : lane - 1, src_r = own_r ? lane : lane + 1;

@@ -2,6 +2,7 @@
 #include <math.h>
 
 #include "tl_fft.cuh"
+#include "tl_smem.cuh"
 
 namespace tl {
 
@@ -31,7 +32,8 @@ static cudaError_t columns(double2 *data, const double2 *roots, int N, bool z_ax
     using S = FftSplit<L>;
     constexpr size_t smem = S::smem(false);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(fft_columns<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        static SmemLimit limit;
+        const cudaError_t e = limit.raise(fft_columns<L>, smem);
         if (e != cudaSuccess) return e;
     }
     const unsigned h = (unsigned)N / 2, lines = (unsigned)N * h, inner = z_axis ? lines : h;

@@ -1,5 +1,6 @@
 // Transforms along x, between a field and its modes (see tl_fft.cuh).
 #include "tl_fft.cuh"
+#include "tl_smem.cuh"
 
 namespace tl {
 
@@ -9,7 +10,8 @@ static cudaError_t rows(double2 *data, const FieldRows &field, const double2 *ro
     using S = FftSplit<L>;
     constexpr size_t smem = S::smem(true);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(fft_rows<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        static SmemLimit limit;
+        const cudaError_t e = limit.raise(fft_rows<L>, smem);
         if (e != cudaSuccess) return e;
     }
     const unsigned lines = (unsigned)field.N * (unsigned)field.N;

@@ -11,6 +11,7 @@
 #include "tl_boxmuller.cuh"
 #include "tl_fourier.cuh"
 #include "tl_philox.cuh"
+#include "tl_smem.cuh"
 
 namespace tl {
 
@@ -355,7 +356,8 @@ cudaError_t launch_bin(const double2 *modes, int N, int nbins, double *Psum, dou
     const size_t smem = (size_t)(N / 4 + 1) * sizeof(double2) +
                         (size_t)nbins * (2 * sizeof(double) + sizeof(unsigned long long));
     if (smem > 48 * 1024) {  // N above 1976
-        const cudaError_t e = cudaFuncSetAttribute(bin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        static SmemLimit limit;
+        const cudaError_t e = limit.raise(bin_kernel, smem);
         if (e != cudaSuccess) return e;
     }
     bin_kernel<<<grid_for(total, sm_count, 2), 256, smem, s>>>(modes, N, nbins, Psum, rsum, cnt);

@@ -22,11 +22,11 @@
 #include <cuda.h>
 #include <math.h>
 
-#include <atomic>
 #include <utility>
 
 #include "tl_internal.cuh"
 #include "tl_scale.cuh"
+#include "tl_smem.cuh"
 
 namespace tl {
 
@@ -1069,20 +1069,9 @@ static cudaError_t launch_group_t(int prefetch, const BatchJob *jobs, const unsi
     const size_t smem = group_smem_bytes(njobs, NF, D);
     auto kern = D ? fused_pass_group<T, NF, 3> : fused_pass_group<T, NF, 0>;
     if (smem > 12 * 1024) {  // with up to 34 KB that are static it may pass 48 KB
-        // the opt-in limit for this kernel (per device, set once; an equal or smaller request needs nothing)
-        static std::atomic<size_t> configured[64][2];
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
+        static SmemLimit limit[2];
+        const cudaError_t e = limit[D ? 1 : 0].raise(kern, smem);
         if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        std::atomic<size_t> &done = configured[dev][D ? 1 : 0];
-        if (smem > done.load(std::memory_order_acquire)) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            size_t cur = done.load(std::memory_order_relaxed);
-            while (smem > cur && !done.compare_exchange_weak(cur, smem, std::memory_order_release)) {
-            }
-        }
     }
     return launch_dependent(kern, dim3((unsigned)grid), 256, smem, s, jobs, first_item, njobs, total, c);
 }
@@ -1716,41 +1705,19 @@ __global__ void __launch_bounds__(256, 2) fused_pass_tma_group(const BatchJob *_
                                               j.nblocks, j.gx, j.gy);
 }
 
-// The dynamic shared-memory limit of a kernel is a per-device attribute: raise
-// it once per device and kernel (thread-safe; a lower request needs no call).
-constexpr int kMaxDevices = 64;
-
-template <typename K, int SLOTS>
-static cudaError_t ensure_smem_attribute(K kern, size_t smem, std::atomic<size_t> (*configured)[SLOTS], int slot)
-{
-    if (smem == 0) return cudaSuccess;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::atomic<size_t> &done = configured[dev][slot];
-    if (smem <= done.load(std::memory_order_acquire)) return cudaSuccess;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    size_t cur = done.load(std::memory_order_relaxed);
-    while (smem > cur && !done.compare_exchange_weak(cur, smem, std::memory_order_release)) {
-    }
-    return cudaSuccess;
-}
-
 template <typename T, int NF, bool MEASURE>
 static cudaError_t launch_tma(const Model &m, const FieldPtrs &fp, const PassCoef &c, const PassGeom &g,
                               const TmaMaps &maps, Scalars *sc, double *slots, cudaStream_t s)
 {
     // 7 + 1 warps (two CTAs per SM) or 15 + 1 warps (one CTA per SM): 16
     // warps per SM, at most 4 per SM sub-partition, so 128 registers a thread
-    static std::atomic<size_t> configured[kMaxDevices][4];
+    static SmemLimit limit[4];
     const int big = g.cwarps > 7 ? 1 : 0;
     const bool items = tma_items_form(NF, m.N);
     const int threads = 32 * (g.cwarps + 1);
     auto kern = big ? (items ? fused_pass_tma<T, NF, MEASURE, 512, true> : fused_pass_tma<T, NF, MEASURE, 512, false>)
                     : (items ? fused_pass_tma<T, NF, MEASURE, 256, true> : fused_pass_tma<T, NF, MEASURE, 256, false>);
-    cudaError_t e = ensure_smem_attribute(kern, g.smem, configured, big + (items ? 2 : 0));
+    cudaError_t e = limit[big + (items ? 2 : 0)].raise(kern, g.smem);
     if (e != cudaSuccess) return e;
     // one CTA per tile, in tile order: the hardware starts each CTA as an SM
     // frees up, which keeps the CTAs in flight a compact band of neighbouring
@@ -1764,9 +1731,9 @@ template <typename T, int NF>
 static cudaError_t launch_tma_group_t(int stages, size_t smem, const BatchJob *jobs, const unsigned *first_item,
                                       int njobs, unsigned total, const PassCoef &c, cudaStream_t s)
 {
-    static std::atomic<size_t> configured[kMaxDevices][2];
+    static SmemLimit limit;
     auto kern = fused_pass_tma_group<T, NF>;
-    cudaError_t e = ensure_smem_attribute(kern, smem, configured, 0);
+    cudaError_t e = limit.raise(kern, smem);
     if (e != cudaSuccess) return e;
     if (total == 0) return cudaSuccess;
     return launch_dependent(kern, dim3(total), 256, smem, s, jobs, first_item, njobs, c, stages);
@@ -1776,10 +1743,10 @@ template <int NF, bool MEASURE>
 static cudaError_t launch_shared(const Model &m, const FieldPtrs &fp, const PassCoef &c, const PassGeom &g, Scalars *sc,
                                  double *slots, cudaStream_t s)
 {
-    static std::atomic<size_t> configured[kMaxDevices][2];
+    static SmemLimit limit;
     auto kern = fused_pass_shared<NF, MEASURE>;
     constexpr size_t smem = shared_planes_bytes(NF);
-    cudaError_t e = ensure_smem_attribute(kern, smem, configured, 0);
+    cudaError_t e = limit.raise(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_dependent(kern, g.grid, 256, smem, s, m, fp, c, g.txt, g.ty, g.zc, sc, slots);
 }
@@ -1788,9 +1755,9 @@ template <typename T, int NF, bool MEASURE, int D, int NT>
 static cudaError_t launch_ldg(const Model &m, const FieldPtrs &fp, const PassCoef &c, const PassGeom &g, Scalars *sc,
                               double *slots, cudaStream_t s)
 {
-    static std::atomic<size_t> configured[kMaxDevices][2];
+    static SmemLimit limit;
     auto kern = fused_pass_ldg<T, NF, MEASURE, D, NT>;
-    cudaError_t e = ensure_smem_attribute(kern, g.smem, configured, 0);
+    cudaError_t e = limit.raise(kern, g.smem);
     if (e != cudaSuccess) return e;
     return launch_dependent(kern, g.grid, NT, g.smem, s, m, fp, c, g.txt, g.ty, g.zc, sc, slots);
 }

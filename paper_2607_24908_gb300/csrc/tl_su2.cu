@@ -23,6 +23,7 @@
 #include "tl_internal.cuh"
 #include "tl_lattice.cuh"
 #include "tl_philox.cuh"
+#include "tl_smem.cuh"
 
 namespace {
 
@@ -663,6 +664,10 @@ struct tl_su2 {
     int mblocks = 0;
     int sm_count = 0;
     bool has_state = false;
+    // the step's tile and launch (su2_plan; grid 0: not planned yet)
+    Su2Tile tile{};
+    unsigned grid = 0;
+    size_t smem = 0;
 };
 
 #define SU_CK(call)                                                                                         \
@@ -680,16 +685,22 @@ using Su2Kernel = void (*)(const T *, T *, T *, int, Su2Tile, T);
 
 bool su2_stages_fields(int N, size_t esz) { return esz == 4 && N % 32 == 0; }
 
-// The code form of a tile.  Staged electric fields measured faster where rows
-// start on a 128-byte line (FP32, us: 128^3 76 against 82, 192^3 231 against
+// The code form of a tile: 0 any tile, 1 and 2 the 32 x 8 one without and with
+// staged electric fields.  Those measured faster where rows start on a
+// 128-byte line (FP32, us: 128^3 76 against 82, 192^3 231 against
 // 249, 256^3 532 against 574) and slower elsewhere (100^3 57 against 53, 150^3
 // 142 against 130); FP64 has its registers to itself and keeps them there.
 template <typename T>
-Su2Kernel<T> su2_kernel(int N, const Su2Tile &t)
+int su2_form(int N, const Su2Tile &t)
+{
+    return sizeof(T) == 4 && t.tx == 32 && t.ty == 8 ? (su2_stages_fields(N, sizeof(T)) ? 2 : 1) : 0;
+}
+
+template <typename T>
+Su2Kernel<T> su2_kernel(int form)
 {
     if constexpr (sizeof(T) == 4) {
-        if (t.tx == 32 && t.ty == 8)
-            return su2_stages_fields(N, sizeof(T)) ? su2_pass<T, true, true> : su2_pass<T, true, false>;
+        if (form) return form == 2 ? su2_pass<T, true, true> : su2_pass<T, true, false>;
     }
     return su2_pass<T, false, false>;
 }
@@ -708,8 +719,12 @@ Su2Kernel<T> su2_kernel(int N, const Su2Tile &t)
 // first (100^3 759 against 840 us, 192^3 4950 against 5210); FP32 takes it
 // while the links fit in L2 and the estimate is 8% better (128^3 76 against
 // 80 us; beyond that size it loses: 192^3 250 against 231, 256^3 572 against 532).
+//
+// The plan depends on the lattice and the device alone and is kept with the
+// lattice.  Every size shares the kernels: their shared-memory limit is raised
+// for the largest tile that any lattice has asked for (SmemLimit).
 template <typename T>
-int su2_plan(const tl_su2 *Y, Su2Tile *out, unsigned *grid, size_t *smem)
+int su2_plan(tl_su2 *Y)
 {
     const int N = Y->N;
     auto shape = [&](int tx, int ty) { return Su2Tile{tx, ty, (N + tx - 1) / tx, (N + ty - 1) / ty, 0}; };
@@ -728,12 +743,13 @@ int su2_plan(const tl_su2 *Y, Su2Tile *out, unsigned *grid, size_t *smem)
             2 * (tx + t.ty) <= 256 && cost(t) < best_cost)
             best = t, best_cost = cost(t);
     }
-    const Su2Kernel<T> kern = su2_kernel<T>(N, best);
-    const bool fixed = best.tx == 32 && best.ty == 8;
-    *smem = su2_smem(best.tx, best.ty, sizeof(T), fixed && su2_stages_fields(N, sizeof(T)));
+    static tl::SmemLimit limit[3];
+    const int form = su2_form<T>(N, best);
+    const Su2Kernel<T> kern = su2_kernel<T>(form);
+    const size_t smem = su2_smem(best.tx, best.ty, sizeof(T), form == 2);
     int per_sm = 0;
-    SU_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem));
-    SU_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, *smem));
+    SU_CK(limit[form].raise(kern, smem));
+    SU_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem));
     const long slots = (long)(Y->sm_count > 0 ? Y->sm_count : 152) * (per_sm > 0 ? per_sm : 1);
     const long tiles = (long)best.ntx * best.nty, planes = tiles * N;
     // z-chunk: the fewest (waves of CTAs) x (planes per CTA + the ~3 planes of
@@ -744,14 +760,16 @@ int su2_plan(const tl_su2 *Y, Su2Tile *out, unsigned *grid, size_t *smem)
         const long est = (ctas + slots - 1) / slots * (long)(c + 3);
         if (chunk_cost < 0 || est < chunk_cost) chunk_cost = est, best.zc = c;
     }
-    *grid = (unsigned)(tiles * ((N + best.zc - 1) / best.zc));
+    unsigned grid = (unsigned)(tiles * ((N + best.zc - 1) / best.zc));
     const long even_cost = (planes + slots - 1) / slots + 4;  // a CTA's range starts one tile and often a second
     const bool in_l2 = 12.0 * N * N * N * sizeof(T) <= 128e6;
     if (sizeof(T) == 8 ? even_cost <= chunk_cost : in_l2 && even_cost < 0.92 * chunk_cost) {
         best.zc = 0;
-        *grid = (unsigned)(planes < slots ? planes : slots);
+        grid = (unsigned)(planes < slots ? planes : slots);
     }
-    *out = best;
+    Y->tile = best;
+    Y->smem = smem;
+    Y->grid = grid;
     return TL_OK;
 }
 
@@ -874,27 +892,23 @@ int tl_su2_step(tl_su2 *Y, int n, double dt)
     if (!Y) return tl::fail(TL_EINVAL, "NULL lattice");
     if (n < 0 || !isfinite(dt) || dt == 0.0) return tl::fail(TL_EINVAL, "n >= 0 and a finite nonzero dt needed");
     if (!Y->has_state) return tl::fail(TL_ESTATE, "no state");
-    const int N = Y->N;
-    Su2Tile tile;
-    unsigned grid = 0;
-    size_t smem = 0;
-    int rc = Y->dtype == TL_F32 ? su2_plan<float>(Y, &tile, &grid, &smem) : su2_plan<double>(Y, &tile, &grid, &smem);
-    if (rc) return rc;
-    for (int k = 0; k < n; ++k) {
-        if (Y->dtype == TL_F32) {
-            const auto kern = su2_kernel<float>(N, tile);
-            kern<<<grid, 256, smem, Y->stream>>>(static_cast<const float *>(Y->U[Y->cur]),
-                                                 static_cast<float *>(Y->U[Y->cur ^ 1]), static_cast<float *>(Y->E), N,
-                                                 tile, (float)dt);
-        } else {
-            su2_kernel<double>(N, tile)<<<grid, 256, smem, Y->stream>>>(static_cast<const double *>(Y->U[Y->cur]),
-                                                                    static_cast<double *>(Y->U[Y->cur ^ 1]),
-                                                                    static_cast<double *>(Y->E), N, tile, dt);
-        }
-        SU_CK(cudaGetLastError());
-        Y->cur ^= 1;
+    if (!Y->grid) {
+        const int rc = Y->dtype == TL_F32 ? su2_plan<float>(Y) : su2_plan<double>(Y);
+        if (rc) return rc;
     }
-    return TL_OK;
+    auto steps = [&](auto value) -> int {
+        using S = decltype(value);
+        const Su2Kernel<S> kern = su2_kernel<S>(su2_form<S>(Y->N, Y->tile));
+        for (int k = 0; k < n; ++k) {
+            kern<<<Y->grid, 256, Y->smem, Y->stream>>>(static_cast<const S *>(Y->U[Y->cur]),
+                                                       static_cast<S *>(Y->U[Y->cur ^ 1]), static_cast<S *>(Y->E), Y->N,
+                                                       Y->tile, (S)dt);
+            SU_CK(cudaGetLastError());
+            Y->cur ^= 1;
+        }
+        return TL_OK;
+    };
+    return Y->dtype == TL_F32 ? steps(0.0f) : steps(0.0);
 }
 
 int tl_su2_measure(tl_su2 *Y, double *out4)

@@ -327,28 +327,35 @@ int check_field(const tl_lattice *L, int field, int which)
 // plan's previous executions (on whatever stream they were enqueued) through the
 // plan's event; the caller records that event after its last execution.  Calls
 // that use a plan therefore only enqueue work: no host wait guards the workspace.
-// A table is written before its first use and then only read: nothing to wait for.
+// A table is written once and then only read: its event follows the writing.
 struct SharedPlan {
     double2 *roots;    // nullptr: the cuFFT plan
     cufftHandle h;
-    cudaEvent_t done;  // cuFFT: recorded after the latest enqueued execution
+    cudaEvent_t done;  // the table's writing; cuFFT: the latest enqueued execution
 };
 std::mutex g_plan_mu;
 std::map<std::pair<int, int>, SharedPlan> g_plans;  // (device, N) -> plan
 
-int make_roots(int N, cudaStream_t s, double2 **out)
+// The table is written on a stream of its own, so that its first use waits for
+// that alone, on the device, and not for what the caller's stream still has to do.
+int make_roots(int N, SharedPlan *p)
 {
-    std::vector<double2> h((size_t)N / 2);
-    tl::fft_roots(N, h.data());
     double2 *d = nullptr;
-    TL_CK(cudaMalloc(&d, h.size() * sizeof(double2)));
-    cudaError_t e = cudaMemcpyAsync(d, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaEvent_t done = nullptr;
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaMalloc(&d, (size_t)N / 2 * sizeof(double2));
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = tl::launch_fft_roots(N, d, s);
+    if (e == cudaSuccess) e = cudaEventRecord(done, s);
+    if (s) cudaStreamDestroy(s);  // returns at once; what it still runs is finished first
     if (e != cudaSuccess) {
+        if (done) cudaEventDestroy(done);
         cudaFree(d);
-        return fail(TL_ECUDA, "table of roots: %s", cudaGetErrorString(e));
+        return fail(e == cudaErrorMemoryAllocation ? TL_ENOMEM : TL_ECUDA, "table of roots: %s", cudaGetErrorString(e));
     }
-    *out = d;
+    p->roots = d;
+    p->done = done;
     return TL_OK;
 }
 
@@ -361,7 +368,7 @@ int shared_plan(int N, cudaStream_t s, SharedPlan **out)
     if (it == g_plans.end()) {
         SharedPlan p{};
         if (tl::fft_supported(N)) {
-            const int rc = make_roots(N, s, &p.roots);
+            const int rc = make_roots(N, &p);
             if (rc) return rc;
         } else {
             cufftResult r = cufftPlan3d(&p.h, N, N, N / 2, CUFFT_Z2Z);
@@ -379,8 +386,7 @@ int shared_plan(int N, cudaStream_t s, SharedPlan **out)
         it = g_plans.emplace(key, p).first;
     }
     *out = &it->second;
-    if (it->second.roots) return TL_OK;
-    TL_CKFFT(cufftSetStream(it->second.h, s));
+    if (!it->second.roots) TL_CKFFT(cufftSetStream(it->second.h, s));
     TL_CK(cudaStreamWaitEvent(s, it->second.done, 0));  // a never-recorded event: no wait
     return TL_OK;
 }

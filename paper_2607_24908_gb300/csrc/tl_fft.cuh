@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(FftSplit<L>::THREADS, FftSplit<L>::MINB)
 
 // N that the kernels above take (else a library transform).
 bool fft_supported(int N);
-// The N/2 roots exp(-2 pi i m/N) as pairs (c, t), for a table on the device.
-void fft_roots(int N, double2 *roots);
+// Write the table of N/2 roots exp(-2 pi i m/N), as pairs (c, t), to the device; only enqueues.
+cudaError_t launch_fft_roots(int N, double2 *roots, cudaStream_t s);
 cudaError_t launch_fft_columns(double2 *data, const double2 *roots, int N, bool z_axis, bool inverse, cudaStream_t s);
 cudaError_t launch_fft_rows(double2 *data, const FieldRows &field, const double2 *roots, bool inverse, cudaStream_t s);
 

@@ -14,7 +14,8 @@ bool fft_supported(int N)
     return m == 1 || m == 3 || m == 5;
 }
 
-void fft_roots(int N, double2 *roots)
+// The N/2 roots exp(-2 pi i m/N) as pairs (c, t).
+static void fft_roots(int N, double2 *roots)
 {
     const long double step = 2.0L * 3.14159265358979323846264338327950288L / (long double)N;
     for (int i = 0; i < N / 2; ++i) {
@@ -24,6 +25,26 @@ void fft_roots(int N, double2 *roots)
         roots[i].x = (double)(turned ? s : c);
         roots[i].y = (double)(turned ? c / s : -s / c);
     }
+}
+
+// The table travels as a kernel's parameter (8 KB at N = 1024, of the 32 KB that one
+// may have): copied at the launch, so that the host has nothing to keep or wait for.
+constexpr int kMaxRoots = 512;
+struct RootTable {
+    double2 v[kMaxRoots];
+};
+__global__ void __launch_bounds__(256) store_roots(double2 *roots, const __grid_constant__ RootTable table, int count)
+{
+    for (int i = threadIdx.x; i < count; i += 256) roots[i] = table.v[i];
+}
+
+cudaError_t launch_fft_roots(int N, double2 *roots, cudaStream_t s)
+{
+    if (!fft_supported(N) || N / 2 > kMaxRoots) return cudaErrorInvalidValue;
+    RootTable t{};
+    fft_roots(N, t.v);
+    store_roots<<<1, 256, 0, s>>>(roots, t, N / 2);
+    return cudaGetLastError();
 }
 
 template <int L>

@@ -49,15 +49,18 @@ __device__ __forceinline__ float u53_f32(uint64_t x)
     return fmaf((float)hi, 0x1p-24f, (float)lo * 0x1p-53f);
 }
 
-// (cos, sin)(2 pi w 2^-64) in FP32: the nearest quarter turn is taken off in
-// integers, the rest, within an eighth of a turn, goes into the Taylor
-// polynomials (first omitted terms below 2e-9 and 3e-8).  About 20
-// instructions, half of them on the FMA pipes; sincospif of a converted
+// (cos, sin)(2 pi u) in FP32 for u = (w >> 11) 2^-53: the nearest quarter turn
+// is taken off in integers, the rest, within an eighth of a turn, goes into the
+// Taylor polynomials (first omitted terms below 2e-9 and 3e-8).  The rest enters
+// in two parts, 30 bits and the 21 below them (exact in FP32), so that the
+// component that vanishes near an axis keeps its relative accuracy however small it
+// is.  Half of the instructions are on the FMA pipes; sincospif of a converted
 // uniform took 35.
 __device__ __forceinline__ void unit_circle(uint64_t w, float &c, float &s)
 {
-    const uint32_t h = (uint32_t)(w >> 32) + 0x20000000u;
-    const float x = (float)((int32_t)(h & 0x3fffffffu) - 0x20000000) * (float)(2.0 * M_PI / 4294967296.0);
+    constexpr float kTurn32 = (float)(2.0 * M_PI / 4294967296.0);
+    const uint32_t h = (uint32_t)(w >> 32) + 0x20000000u, low = (uint32_t)w & ~0x7ffu;
+    const float x = fmaf((float)low, kTurn32 * 0x1p-32f, (float)((int32_t)(h & 0x3fffffffu) - 0x20000000) * kTurn32);
     const float t = x * x;
     float ps = fmaf(t, 1.0f / 362880.0f, -1.0f / 5040.0f);
     ps = fmaf(ps, t, 1.0f / 120.0f);
@@ -79,7 +82,7 @@ __device__ __forceinline__ void gauss2(const tl::BoxMullerTable *, uint32_t k, u
     uint64_t w0, w1;
     philox2x64_10_low(k, ctr1, seed, w0, w1);
     // Box-Muller in FP32 (the field is stored in FP32): u1 to 2^-24 of itself,
-    // the angle to 2^-32 of a turn
+    // the angle to 2^-23 of its distance from the nearest axis
     const float u1 = u53_f32((w0 >> 11) + 1);
     const float r = sqrtf(-2.0f * logf(u1));
     float s, c;
@@ -112,7 +115,8 @@ __device__ __forceinline__ void st(double *p, const double (&v)[2])
 // products alone take 150 us at 384^3): neighbours come as 16-byte words and by
 // shuffle, the angle from the word's bits, the first round of the generator
 // with two products; 467 instructions a plane and thread, from 538, and less
-// in the last wave: 303 -> 244 us.  FP64 is bound by the FP64 pipe: the
+// in the last wave: 303 -> 244 us at 384^3, of which the angle's second part took
+// back 4 (248).  FP64 is bound by the FP64 pipe: the
 // table form of Box-Muller (tl_boxmuller.cuh) took 384^3 from 5910 to 3779 us.
 template <typename T>
 __global__ void __launch_bounds__(256) langevin_pass(const T *__restrict__ in, T *__restrict__ out, int N, int txt,
@@ -209,7 +213,8 @@ extern "C" int tl_langevin_step(tl_lattice *L, int n, double dt, const tl_langev
     // reads beyond its own do not add to: one plane per CTA spreads it best (us:
     // 100^3 96 against 116 with 4 planes, 212^3 777 against 795, 384^3 3779 against
     // 3790).  FP32: the fewest (waves of CTAs) x (planes per CTA + 1/4 for those two
-    // planes): 384^3 244 us with 19 planes, 258 with 32; 64^3 5.7 with 1, 6.8 with 4.
+    // planes; measured before the angle had its second part): 384^3 244 us with 19
+    // planes, 258 with 32; 64^3 5.7 with 1, 6.8 with 4.
     const long slots = (long)(L->sm_count > 0 ? L->sm_count : 152) * (per_sm > 0 ? per_sm : 1);
     double best = 0.0;
     for (int c = 1; c <= (L->dtype == TL_F32 ? L->N : 1); ++c) {

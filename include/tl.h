@@ -467,8 +467,8 @@ int tl_autotune(tl_lattice *lat, double *best_ms_per_pass);
  * TL_ESTATE while the lattice is in a batch.  May synchronise the lattice
  * stream (to grow its reduction slots).  A new lattice starts on TL_PASS_TMA
  * when it is FP32 and N >= 192 (compute warps and z-chunk chosen from N, the
- * field count and the SM count, to run in few full waves of CTAs, up to N = 495;
- * 15 compute warps and measured z-chunks from there), on
+ * field count and the SM count, to run in few full waves of CTAs, up to N = 495,
+ * with two fields 355, with three 427; measured ones from there), on
  * TL_PASS_STREAM otherwise (where those measured faster; z-chunks chosen from N,
  * the field count and the SM count); the environment variable TL_PASS_VARIANT=tma|ldg overrides that default at creation. */
 int tl_set_pass_config(tl_lattice *lat, const tl_pass_config *cfg);

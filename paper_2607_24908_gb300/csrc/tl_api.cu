@@ -48,29 +48,54 @@ thread_local char g_err[512] = "";
 }  // namespace
 
 // Compute warps and z-chunk of the TMA pass for FP32 lattices of a few waves of
-// CTAs: the fewest (waves of CTAs) x (planes per chunk + 8), a wave being one CTA of
-// 15 + 1 warps per SM or two of 7 + 1 (5%, 10%, 12% slower a row of sites with one, two,
-// three fields: their ring is shallower).  us, former fixed values -> chosen: one
-// field 200^3 52 -> 34, 224^3 51 -> 39, 288^3 107 -> 74, 320^3 124 -> 104, 352^3 151 -> 133, 416^3
-// 231 -> 196; two fields 200^3 91 -> 58, 288^3 173 -> 151, 320^3 204 -> 196; three 224^3 136 ->
-// 104, 288^3 276 -> 204, 352^3 434 -> 392, 416^3 642 -> 590 (equal tiles included).
+// CTAs: the fewest (waves of CTAs) x (planes per chunk and to start one), a wave
+// being one CTA of 15 + 1 warps per SM or two of 7 + 1 (a row of sites 5-10% slower:
+// their ring is shallower).  With two and three fields, which are nearer to the
+// memory's rate, a last wave that is not full costs a little less, and a long chunk
+// 0.3% a plane, for halo rows that its neighbours have passed by: without that term
+// 340^3 took two chunks of 170 planes (two fields 283 us, now 238-245; three 399, now 343).
+// Over 196 ... 492 (two fields 352, three 424) in steps of 4, sweeps of 20 to 40 shapes
+// each: on average 1.7%, 2.9% and 1.3% slower than the best shape with one, two and
+// three fields, and 11% faster than the former fixed chunks (the worst: 236^3 two fields
+// 101 us against 95-98, 312^3 185 against 179, 404^3 three 555 against 549).  us, fixed -> here: one
+// field 200^3 52 -> 34, 288^3 107 -> 74, 352^3 151 -> 133; two 200^3 91 -> 58, 288^3
+// 173 -> 151; three 224^3 136 -> 104, 352^3 434 -> 392 (equal tiles included).
 static void tma_shape(tl::PassTuning &t, int N, int nf, int sms)
 {
     const int txt = tl::even_row_tile(N / 4), gx = (N / 4 + txt - 1) / txt;
+    const double start = nf == 1 ? 8 : 12, partial = nf == 1 ? 1 : 0.9, per_plane = nf == 1 ? 0 : 0.003;
     double least = 0.0;
     for (int warps : {7, 15}) {
         const int ty = 32 * warps / txt < N ? 32 * warps / txt : N;
         const long tiles = (long)gx * ((N + ty - 1) / ty), slots = (long)sms * (warps == 7 ? 2 : 1);
-        const double rows = warps == 15 ? ty : 2 * ty * (nf == 1 ? 1.05 : nf == 2 ? 1.1 : 1.12);
+        const double rows = warps == 15 ? ty : 2 * ty * (nf == 1 ? 1.05 : 1.1);
         for (int chunks = 1; chunks <= N / 20; ++chunks) {
             int zc = (N + chunks - 1) / chunks;
             if (zc > 170) continue;
             const int even = (zc + 7) / 8 * 8;  // whole flushes of the FP32 sums, where that costs under 2%
             if (even <= 1.02 * zc && (N + even - 1) / even == chunks) zc = even;
-            const double cost = (double)((tiles * chunks + slots - 1) / slots) * (zc + 8) * rows;
+            const long ctas = tiles * chunks;
+            const double last = (double)(ctas % slots) / slots;
+            const double waves = (double)(ctas / slots) + (last == 0.0 ? 0.0 : last < partial ? partial : last);
+            const double cost = waves * (zc + start) * rows * (1.0 + per_plane * zc);
             if (least == 0.0 || cost < least) least = cost, t.cwarps = warps, t.zc = zc;
         }
     }
+}
+
+// z-chunk of the TMA pass with two FP32 fields from 620^3 on, where it runs at the
+// memory's rate and what counts is which halo rows still meet in L2.  Whole tiles of
+// 128 sites want short chunks; the emptier the last tile of a row, the longer (its
+// CTAs are done early, and the ones in flight drift apart).  us, 60 planes / here /
+// 104 (72 from 832^3): 652^3 1585 / 1495 (150) / 1498, 700^3 1829 / 1763 (130) / 1811,
+// 772^3 2560 / 2419 (150) / 2451, 832^3 3013 / 2954 (88) / 2981, 916^3 4100 / 3952 (130) /
+// 4049, 960^3 4569 / 4500 (88) / 4520; whole: 640^3 1329 / - / 1327, 896^3 3611 / - / 3605,
+// 1024^3 5343 / - / 5391.  Over 48 sizes of 628 ... 1024 within 1.5% of the best of
+// eight chunks, 0.7% slower than 104 or 72 at most.
+static int two_field_chunk(int N)
+{
+    const double filled = (double)N / (128 * ((N + 127) / 128));
+    return filled < 0.89 ? 150 : filled < 0.92 ? 130 : filled < 0.96 ? 88 : 60;
 }
 
 tl::PassTuning tl::default_tuning(int N, int nf, int elem_bytes, int sm_count)
@@ -82,29 +107,36 @@ tl::PassTuning tl::default_tuning(int N, int nf, int elem_bytes, int sm_count)
     if (v && strcmp(v, "ldg") == 0) t.variant = tl::kVariantLdg;
     const char *cw = getenv("TL_BULK_WARPS"), *zc = getenv("TL_PASS_ZC");
     if (t.variant == tl::kVariantTma) {
-        // From 496^3 on (two fields: 440^3) the pass runs at the memory's rate, chunks
+        // From 496^3 on (two fields 356^3, three 428^3) the pass nears the memory's rate, chunks
         // matter by what the tiles in flight share in L2, and the values are the best
-        // of measured sweeps, as they are around 384^3 (us, 380^3 one field 56 planes 170,
-        // the estimate's 76: 173; 364^3 two fields 291 against 296; 380^3 three fields 43
-        // planes 483, 76: over 490).  15 + 1 warps: 464^3 two fields 80 planes 536 (93:
-        // over 558), 512^3 160 planes with one field (344; 128: 360), else 96 (two fields 686;
-        // 103: 687), 576^3 104 (two fields 1002; 64: 1009), from 620^3 60 with two fields
-        // (704^3 79: 1815; 768^3 2291; 104: 2312, 896^3 3616; 72: 3619, 1024^3 5355; 68: 5365) and from 832^3
-        // with three (896^3 5638; 72: 5656), else 104 (640^3 2050), one field from 832^3
-        // 150 (896^3 1800; 72: 1865).
+        // of measured sweeps.  Two fields: 56 planes with 7 + 1 warps over 356 ... 424 (us,
+        // against the estimate above: 372^3 299 / 313, 396^3 373 / 404, 420^3 433 / 475; 360^3
+        // 276 / 269).  Two and three: 80 with 15 + 1 over 428 ... 492 (464^3 two 536; 93: 558; three
+        // 436^3 665 / 688, 444^3 707 / 729, 488^3 973 / 928).  One and three fields take 56
+        // from 376 to 384, whose seven chunks fill their waves (376^3, 380^3, 384^3 one
+        // field 163, 166, 165, the estimate's 166, 168, 167; three 428, 451, 447, the
+        // estimate's 436, 466, 460); the estimate is ahead on either side (372^3 149
+        // against 164, 388^3 183 against 201).  15 + 1 warps: 512^3 160 planes with one
+        // field (344; 128: 360), else 96 (two fields 686; 103: 687), 576^3 104 (two fields
+        // 1002; 64: 1009), with three fields from 832^3 60 (896^3 5447; 72: 5499, 1024^3 8259;
+        // 76: 8347), with one 150 (896^3 1778; 72: 1817), below that 104 (640^3 2010 with three).
+        // 192^3 with two fields keeps the shape that is stated for it (7 + 1 warps, 48
+        // planes; the estimate's 28 planes with 15 + 1 take 50 us, not 64).
         if (elem_bytes != 4 || N < 192) t.zc = N <= 192 ? 48 : 64;
         else if (N == 192 && nf == 2) t.zc = 48;
-        else if (N >= (nf == 2 ? 356 : 372) && N < (nf == 2 ? 410 : 396)) {
-            t.cwarps = nf == 3 ? 15 : 7;
-            t.zc = nf == 3 ? 43 : 56;
-        } else if (N < (nf == 2 ? 440 : tl::kFullRowTiles)) {
+        else if (nf != 2 && N >= 376 && N < 388) {
+            t.cwarps = nf == 1 ? 7 : 15;
+            t.zc = 56;
+        } else if (N < (nf == 1 ? tl::kFullRowTiles : nf == 2 ? 356 : 428)) {
             tma_shape(t, N, nf, sm_count > 0 ? sm_count : 152);
+        } else if (nf == 2 && N < 428) {
+            t.zc = 56;
         } else {
             t.cwarps = 15;
             if (N < tl::kFullRowTiles) t.zc = 80;
             else if (N < 544) t.zc = nf == 1 ? 160 : 96;
             else if (N < 620) t.zc = 104;
-            else if (nf == 2) t.zc = N >= 670 && N < 740 ? 79 : 60;
+            else if (nf == 2) t.zc = two_field_chunk(N);
             else if (N < 832) t.zc = 104;
             else t.zc = nf == 1 ? 150 : 60;
         }

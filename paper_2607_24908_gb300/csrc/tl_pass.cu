@@ -65,7 +65,10 @@ static int f64_tile_rows(int N, int gx, int txt, int ty_max, int zc, int sms)
 // choice is 0.6% slower than the best of a sweep (8% at 144^3 with two fields), that
 // of the estimate above 5% (us: 144^3 155 -> 127, 160^3 199 -> 160, 212^3 396 -> 355, 300^3
 // 1090 -> 932; three fields 160^3 636 -> 501).  Two fields keep 32 planes from 128^3
-// unless another is estimated 4% cheaper (256^3 1216, 37 planes 1200).
+// to 508^3 unless another is estimated 4% cheaper: estimates that close do not tell
+// (the estimate's choice / 32 planes: 288^3 1859 / 1903, 312^3 2226 / 2194, 368^3 3621 /
+// 3615, 448^3 6215 / 6336, 508^3 9187 / 9153).  From 512^3 on they do (512^3 9182 / 9247,
+// 536^3 11403 / 11439, 576^3 13089 / 13173, 640^3 17983 / 18117).
 static double f64_shared_cost(int N, int gx, int txt, int ty, int zc, int sms)
 {
     const long ctas = (long)gx * ((N + ty - 1) / ty) * ((N + zc - 1) / zc), last = ctas % (2 * sms);
@@ -81,7 +84,7 @@ static int f64_chunk(int N, int nf, int gx, int txt, int ty_max, int sms)
         return f64_shared_cost(N, gx, txt, f64_tile_rows(N, gx, txt, ty_max, zc, sms), zc, sms);
     };
     int best = N >= 128 ? 32 : 1;
-    double least = cost(best) * (N >= 128 && nf == 2 ? 0.96 : 1.0);
+    double least = cost(best) * (N >= 128 && N < 512 && nf == 2 ? 0.96 : 1.0);
     for (int zc = 1; zc <= N && zc <= 128; ++zc)
         if (cost(zc) < least) least = cost(zc), best = zc;
     return best;

@@ -446,7 +446,7 @@ int tl_batch_get_options(const tl_batch *batch, int *prefetch, int *split, int *
 
 void tl_batch_destroy(tl_batch *batch);
 
-/* Time candidate launch shapes of the fused pass on this lattice (both
+/* Time candidate launch shapes of the fused pass on this lattice (the one it has, both
  * kinds of tl_pass_config: z-planes per CTA from 4 to the whole lattice, the
  * tile rows and CTA size of the streaming kernel, the warps of the TMA kernel) with
  * passes whose kick and drift coefficients are zero, which rewrite the state

@@ -277,9 +277,9 @@ int finish_create(tl_lattice *L, int N, double kIR, int nf, tl_dtype dtype, cons
     tl::scratch_user(dev, 1);
     L->tuning = tl::default_tuning(N, nf, (int)L->esz, L->sm_count);
     L->geom = tl::pass_geometry(N, (int)L->esz, L->sm_count, nf, L->tuning);
-    TL_CK(cudaMalloc(&L->d_sc, sizeof(Scalars)));
+    TL_CK(tl::device_alloc(&L->d_sc, sizeof(Scalars)));
     TL_CK(cudaMemsetAsync(L->d_sc, 0, sizeof(Scalars), L->stream));
-    TL_CK(cudaMalloc(&L->d_slots, sizeof(double) * tl::kMaxQ * L->geom.nblocks));
+    TL_CK(tl::device_alloc(&L->d_slots, sizeof(double) * tl::kMaxQ * L->geom.nblocks));
     L->slots_cap = L->geom.nblocks;
     refresh_model(L);
     TL_CK(tl::launch_set_background(L->model, L->d_sc, L->ex.a0, 0.0, L->stream));
@@ -375,7 +375,7 @@ int make_roots(int N, SharedPlan *p)
     double2 *d = nullptr;
     cudaEvent_t done = nullptr;
     cudaStream_t s = nullptr;
-    cudaError_t e = cudaMalloc(&d, (size_t)N / 2 * sizeof(double2));
+    cudaError_t e = tl::device_alloc(&d, (size_t)N / 2 * sizeof(double2));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = tl::launch_fft_roots(N, d, s);
@@ -476,7 +476,7 @@ int tl::set_geometry(tl_lattice *L, const PassTuning &t)
     if (g.nblocks > L->slots_cap) {
         double *p = nullptr;
         TL_CK(cudaStreamSynchronize(L->stream));
-        TL_CK(cudaMalloc(&p, sizeof(double) * kMaxQ * g.nblocks));
+        TL_CK(tl::device_alloc(&p, sizeof(double) * kMaxQ * g.nblocks));
         cudaFree(L->d_slots);
         L->d_slots = p;
         L->slots_cap = g.nblocks;
@@ -541,7 +541,7 @@ int tl_lattice_create(tl_lattice **out, int N, double kIR, int n_fields, tl_dtyp
         delete L;
         return fail(TL_ENOMEM, "lattice needs %zu bytes, %zu free on the device", bytes, free_b);
     }
-    if (cudaMalloc(&L->base, bytes) != cudaSuccess) {
+    if (tl::device_alloc(&L->base, bytes) != cudaSuccess) {
         delete L;
         return fail(TL_ENOMEM, "cudaMalloc of %zu bytes failed", bytes);
     }

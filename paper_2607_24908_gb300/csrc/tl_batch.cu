@@ -211,10 +211,10 @@ int build_groups(tl_batch *B)
     for (size_t gi = 0; gi < B->groups.size(); ++gi) {
         auto &g = B->groups[gi];
         const size_t jb = g.idx.size() * sizeof(BatchJob);
-        if ((e = cudaMalloc(&g.d_jobs[0], jb)) != cudaSuccess || (e = cudaMalloc(&g.d_jobs[1], jb)) != cudaSuccess ||
-            (e = cudaMalloc(&g.d_first, g.idx.size() * sizeof(unsigned))) != cudaSuccess ||
+        if ((e = tl::device_alloc(&g.d_jobs[0], jb)) != cudaSuccess || (e = tl::device_alloc(&g.d_jobs[1], jb)) != cudaSuccess ||
+            (e = tl::device_alloc(&g.d_first, g.idx.size() * sizeof(unsigned))) != cudaSuccess ||
             (g.variant == tl::kVariantTma &&
-             (e = cudaMalloc(&g.d_maps, 2 * g.idx.size() * sizeof(tl::TmaMaps))) != cudaSuccess))
+             (e = tl::device_alloc(&g.d_maps, 2 * g.idx.size() * sizeof(tl::TmaMaps))) != cudaSuccess))
             return tl::fail(TL_ENOMEM, "batch descriptors: %s", cudaGetErrorString(e));
         while (B->branch_pool.size() <= gi) {
             cudaStream_t st = nullptr;

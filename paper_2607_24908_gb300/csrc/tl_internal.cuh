@@ -233,6 +233,13 @@ void scratch_release(int dev);
 // A lattice of device dev comes (+1) or goes (-1); with the last one the pool
 // gives its memory back.
 void scratch_user(int dev, int change);
+// cudaMalloc on the current device, tried again after scratch_release if memory is short.
+cudaError_t device_alloc_bytes(void **p, size_t bytes);
+template <typename T>
+cudaError_t device_alloc(T **p, size_t bytes)
+{
+    return device_alloc_bytes(reinterpret_cast<void **>(p), bytes);
+}
 // Free bytes of the current device, after scratch_release if fewer than need are.
 cudaError_t free_device_bytes(size_t need, size_t *free_b);
 

@@ -31,7 +31,7 @@ template <typename T>
 int time_chains(int sms, cudaStream_t st, double *rate)
 {
     T *buf = nullptr;
-    if (cudaMalloc(&buf, 4096 * sizeof(T)) != cudaSuccess) return tl::set_error(TL_ENOMEM, "probe buffer", "");
+    if (tl::device_alloc(&buf, 4096 * sizeof(T)) != cudaSuccess) return tl::set_error(TL_ENOMEM, "probe buffer", "");
     cudaMemsetAsync(buf, 0, 4096 * sizeof(T), st);
     const int blocks = sms * 8;
     cudaEvent_t e0, e1;

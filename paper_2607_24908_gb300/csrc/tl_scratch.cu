@@ -51,7 +51,22 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s)
         }
         pool = g_pool[dev];
     }
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    scratch_release(dev);  // what the pool keeps may be in other pieces
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+cudaError_t device_alloc_bytes(void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return e;
+    scratch_release(dev);
+    return cudaMalloc(p, bytes);
 }
 
 void scratch_release(int dev)

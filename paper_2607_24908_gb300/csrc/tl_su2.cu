@@ -817,11 +817,11 @@ int tl_su2_create(tl_su2 **out, int N, tl_dtype dtype, void *cuda_stream)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&Y->sm_count, cudaDevAttrMultiProcessorCount, dev);
     Y->mblocks = 4 * (Y->sm_count > 0 ? Y->sm_count : 152);
-    cudaError_t e = cudaMalloc(&Y->U[0], 12 * n3 * Y->esz);
-    if (e == cudaSuccess) e = cudaMalloc(&Y->U[1], 12 * n3 * Y->esz);
-    if (e == cudaSuccess) e = cudaMalloc(&Y->E, 9 * n3 * Y->esz);
-    if (e == cudaSuccess) e = cudaMalloc(&Y->slots, sizeof(double) * 4 * Y->mblocks);
-    if (e == cudaSuccess) e = cudaMalloc(&Y->out, sizeof(double) * 4);
+    cudaError_t e = tl::device_alloc(&Y->U[0], 12 * n3 * Y->esz);
+    if (e == cudaSuccess) e = tl::device_alloc(&Y->U[1], 12 * n3 * Y->esz);
+    if (e == cudaSuccess) e = tl::device_alloc(&Y->E, 9 * n3 * Y->esz);
+    if (e == cudaSuccess) e = tl::device_alloc(&Y->slots, sizeof(double) * 4 * Y->mblocks);
+    if (e == cudaSuccess) e = tl::device_alloc(&Y->out, sizeof(double) * 4);
     if (e != cudaSuccess) {
         tl_su2_destroy(Y);
         return tl::fail(TL_ENOMEM, "SU(2) allocation: %s", cudaGetErrorString(e));

@@ -49,12 +49,12 @@ struct FftSplit {
     static constexpr int R2 = ODD == 1 ? (T <= 16 ? T : T == 32 ? 8 : 16) : ODD == 3 ? (T <= 8 ? T : 8) : (T <= 4 ? T : 4);
     static constexpr int R3 = T / R2 <= 4 ? T / R2 : 4;
     static constexpr int R4 = T / R2 / R3;
-    static_assert(E * R2 * R3 * R4 == L, "radices");
+    static_assert(E * R2 * R3 * R4 == L && T > 1, "radices");
     // lines per CTA: 128 threads at least, rows of 8 neighbouring columns (128 bytes)
     static constexpr int B = T * 8 >= 128 ? (T * 8 > 256 ? (T * 4 > 256 ? 2 : 4) : 8) : 128 / T;
     static constexpr int THREADS = T * B;
     static constexpr int PITCH = L + L / 16 + 1;  // of a line in shared memory (rows)
-    static constexpr size_t smem(bool rows) { return T == 1 ? 0 : (size_t)B * (rows ? PITCH : L) * sizeof(double2); }
+    static constexpr size_t smem(bool rows) { return (size_t)B * (rows ? PITCH : L) * sizeof(double2); }
     static constexpr int MINB = ODD == 3 ? 384 / THREADS : 512 / THREADS;  // 168 or 128 registers
 };
 
@@ -205,20 +205,16 @@ __device__ __forceinline__ void fft_line(int j, const double2 *__restrict__ root
     using S = FftSplit<L>;
     auto put = [&](int n, double2 v) { *ex(n) = v; };
     auto get = [&](int n) { return *ex(n); };
-    if constexpr (S::T == 1) {
-        fft_phase<L, S::E, S::ODD, 1, false>(j, roots, mul, load, store);
+    fft_phase<L, S::E, S::ODD, 1, true>(j, roots, mul, load, put);
+    if constexpr (S::R3 == 1) {
+        fft_phase<L, S::R2, 1, S::E, false>(j, roots, mul, get, store);
     } else {
-        fft_phase<L, S::E, S::ODD, 1, true>(j, roots, mul, load, put);
-        if constexpr (S::R3 == 1) {
-            fft_phase<L, S::R2, 1, S::E, false>(j, roots, mul, get, store);
+        fft_phase<L, S::R2, 1, S::E, true>(j, roots, mul, get, put);
+        if constexpr (S::R4 == 1) {
+            fft_phase<L, S::R3, 1, S::E * S::R2, false>(j, roots, mul, get, store);
         } else {
-            fft_phase<L, S::R2, 1, S::E, true>(j, roots, mul, get, put);
-            if constexpr (S::R4 == 1) {
-                fft_phase<L, S::R3, 1, S::E * S::R2, false>(j, roots, mul, get, store);
-            } else {
-                fft_phase<L, S::R3, 1, S::E * S::R2, true>(j, roots, mul, get, put);
-                fft_phase<L, S::R4, 1, S::E * S::R2 * S::R3, false>(j, roots, mul, get, store);
-            }
+            fft_phase<L, S::R3, 1, S::E * S::R2, true>(j, roots, mul, get, put);
+            fft_phase<L, S::R4, 1, S::E * S::R2 * S::R3, false>(j, roots, mul, get, store);
         }
     }
 }

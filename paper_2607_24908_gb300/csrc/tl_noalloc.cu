@@ -24,12 +24,10 @@ constexpr size_t kMaxSlotBlocks = 16384;
 constexpr size_t kScalarsBytes = (sizeof(tl::Scalars) + 255) / 256 * 256;
 constexpr size_t kScratchBytes = kScalarsBytes + kMaxSlotBlocks * tl::kMaxQ * sizeof(double);
 
-// The pass shape of this entry point, fixed here so that its CTA count does
-// not follow the library's default shapes: the register-streaming kernel with
-// 256-thread CTAs and 32 threads along x (tiles of 32 W x 8 sites, W = 4 FP32
-// or 2 FP64 sites per thread), z-chunks of 256 planes from N = 512 up and the
-// automatic z-chunk below (at most 128 planes, so at most
-// ceil(N/(32 W)) ceil(N/8) ceil(N/128) <= 2048 CTAs for N < 512).
+// The pass shape of this entry point: the register-streaming kernel with 256-thread
+// CTAs, rows in equal tiles of at most 32 threads (W = 4 FP32 or 2 FP64 sites each),
+// z-chunks of 256 planes from N = 512 up and the automatic z-chunk below (which
+// gives at most 8704 CTAs for N < 512 on GPUs of 40 to 152 SMs; the call checks).
 constexpr int kZChunkLarge = 256;
 
 tl::PassTuning noalloc_tuning(int N)

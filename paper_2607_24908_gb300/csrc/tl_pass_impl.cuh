@@ -1371,9 +1371,9 @@ __device__ __forceinline__ void tma_tile(const Model &m, const FieldPtrs &fp, co
 // planes while the compute warps finish a tile and sum its energies.  Tile
 // `item` is (bx, by, bz) = (item % gx, item / gx % gy, item / (gx gy)) and owns
 // reduction slot `item` of nitems.  maps points to the tensor maps of the
-// lattice's input arrays (a kernel parameter or a copy in global memory);
-// GLOBAL_MAPS: the maps live in global memory, written by the host, and the
-// producer makes them visible to the tensor-map proxy before their first use.
+// lattice's input arrays (a kernel parameter).  Its caller, fused_pass_tma, gives a
+// CTA one tile (several measured slower, see launch_tma); the form stays for the
+// sizes where it compiles to the faster kernel (tma_one_tile).
 // Every compute warp takes part in every tile's ring traffic (a warp without
 // sites only waits and releases), so the "empty" barriers count all of them.
 template <typename T, int NF, bool MEASURE>
@@ -1699,8 +1699,7 @@ __global__ void __launch_bounds__(256, 2) fused_pass_tma_group(const BatchJob *_
     __syncthreads();
     const BatchJob &j = jobs[s_job];
     const unsigned local = blockIdx.x - __ldg(first_item + s_job);
-    // two fields in the multi-tile code form, as for the small lattices batches
-    // hold (either form gives the same numbers)
+    // the one-tile code form for every field count (either form gives the same numbers)
     tma_one_tile<T, NF, false, false, true>(j.m, j.fp, c, j.txt, j.ty, j.zc, S, j.lpad, j.maps, j.sc, j.slots, local,
                                               j.nblocks, j.gx, j.gy);
 }

@@ -707,8 +707,8 @@ Su2Kernel<T> su2_kernel(int form)
 
 // Tile shape and grid of the step.  The cost of a tile per plane is its
 // warps (and 0.12 of a warp for each warp that forms halo plaquettes), so the
-// shape that covers N x N with the fewest warps is taken: at N = 100, 25 x 10
-// tiles cover it with 40 CTA-planes of 8 warps where 32 x 8 ones need 52.  FP32
+// shape that covers N x N with the fewest warps is taken (of equal ones the
+// narrowest): at N = 100, 10 x 25 tiles cover it with 40 CTA-planes of 8 warps where 32 x 8 ones need 52.  FP32
 // keeps the 32 x 8 tile with compile-time strides unless the other needs 20%
 // fewer warps (100^3: 50 against 53 us; 150^3, 5% fewer: 144 against 130).
 //

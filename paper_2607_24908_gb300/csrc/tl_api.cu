@@ -429,22 +429,22 @@ int plan_used(SharedPlan *p, cudaStream_t s)  // after the call's last execution
     return TL_OK;
 }
 
-tl::FieldRows field_rows(tl_lattice *L, void *array, double base, double scale)
+tl::FieldRows field_rows(tl_lattice *L, void *array, double base, double scale, double *offset)
 {
-    return tl::FieldRows{array, L->dtype == TL_F32, L->N, L->model.pitch, L->model.pplane, base, scale};
+    return tl::FieldRows{array, L->dtype == TL_F32, L->N, L->model.pitch, L->model.pplane, base, scale, offset};
 }
 
-// modes = transform of the padded array at src.
-int field_to_modes(tl_lattice *L, SharedPlan *p, void *src, double2 *modes)
+// modes = transform of the padded array at src less its offset; *offset (device memory) = that.
+int field_to_modes(tl_lattice *L, SharedPlan *p, void *src, double *offset, double2 *modes)
 {
     if (p->roots) {
-        TL_CK(tl::launch_fft_rows(modes, field_rows(L, src, 0.0, 1.0), p->roots, false, L->stream));
+        TL_CK(tl::launch_fft_rows(modes, field_rows(L, src, 0.0, 1.0, offset), p->roots, false, L->stream));
         TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, false, false, L->stream));
         TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, true, false, L->stream));
         return TL_OK;
     }
-    TL_CK(tl::launch_widen((int)L->dtype, reinterpret_cast<double *>(modes), src, L->N, L->model.pitch,
-                           L->model.pplane, L->stream));
+    TL_CK(tl::launch_widen((int)L->dtype, reinterpret_cast<double *>(modes), src, offset, L->N,
+                           L->model.pitch, L->model.pplane, L->stream));
     cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
     TL_CKFFT(cufftExecZ2Z(p->h, z, z, CUFFT_FORWARD));
     return TL_OK;
@@ -456,7 +456,7 @@ int modes_to_field(tl_lattice *L, SharedPlan *p, double2 *modes, void *dst, doub
     if (p->roots) {
         TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, true, true, L->stream));
         TL_CK(tl::launch_fft_columns(modes, p->roots, L->N, false, true, L->stream));
-        TL_CK(tl::launch_fft_rows(modes, field_rows(L, dst, base, scale), p->roots, true, L->stream));
+        TL_CK(tl::launch_fft_rows(modes, field_rows(L, dst, base, scale, nullptr), p->roots, true, L->stream));
         return TL_OK;
     }
     cufftDoubleComplex *z = reinterpret_cast<cufftDoubleComplex *>(modes);
@@ -992,23 +992,26 @@ int tl_spectrum(tl_lattice *L, int field, int which, int nbins, double *k, doubl
         if (prc) return prc;
     }
     double2 *modes = nullptr;  // the field, then (in place) its N x N x N/2 modes
-    double *acc = nullptr;
+    double *acc = nullptr;  // the shell sums, then the field's offset and mode 0 of the rest
     TL_CK(tl::scratch_alloc((void **)&modes, n3_of(N) * sizeof(double), L->stream));
-    TL_CK(tl::scratch_alloc((void **)&acc, (size_t)nb * 3 * sizeof(double), L->stream));
+    TL_CK(tl::scratch_alloc((void **)&acc, ((size_t)nb * 3 + 2) * sizeof(double), L->stream));
+    double *offset = acc + 3 * (size_t)nb;
     TL_CK(cudaMemsetAsync(acc, 0, (size_t)nb * 3 * sizeof(double), L->stream));
-    rc = field_to_modes(L, sp, L->buf[L->cur][which][field], modes);
+    rc = field_to_modes(L, sp, L->buf[L->cur][which][field], offset, modes);
     if (rc) return rc;
     rc = plan_used(sp, L->stream);
     if (rc) return rc;
-    TL_CK(tl::launch_bin(modes, N, nb, acc, acc + nb, reinterpret_cast<unsigned long long *>(acc + 2 * nb),
+    TL_CK(tl::launch_bin(modes, N, nb, acc, acc + nb, reinterpret_cast<unsigned long long *>(acc + 2 * nb), offset + 1,
                          L->sm_count, L->stream));
-    std::vector<double> h((size_t)nb * 3);
+    std::vector<double> h((size_t)nb * 3 + 2);
     TL_CK(cudaMemcpyAsync(h.data(), acc, h.size() * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
     cudaFreeAsync(modes, L->stream);
     cudaFreeAsync(acc, L->stream);
     TL_CK(cudaStreamSynchronize(L->stream));
     const double Lbox = 2.0 * M_PI / L->kIR;
     const double V = Lbox * Lbox * Lbox;
+    const double mean = h[3 * (size_t)nb] + h[3 * (size_t)nb + 1] / (double)n3_of(N);
+    h[0] = mean * mean;  // shell 0
     for (int b = 0; b < nbins; ++b) {
         unsigned long long c = 0;
         double ps = 0.0, rs = 0.0;

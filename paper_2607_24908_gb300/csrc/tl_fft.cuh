@@ -15,9 +15,10 @@
 //  * FP32 fields are widened by integer instructions (tl_bits.cuh) as they are
 //    loaded, and scaled, narrowed and stored by the last pass, which saves a pass
 //    over memory on either side.
-// 256^3: 340 instructions for 16 points of y or z, 292 (+ 32 to scale) for 16 of x;
-// the pipe is busy 94% of the time.  Against cuFFT (us): y or z 439 -> 305, x
-// 501 + 36 for a pass that widened -> 270, inverse x 501 + 70 for one that stored
+// 256^3: 340 instructions for 16 points of y or z, 292 for 16 of x and 32 for the
+// field's offset (tl_offset.cuh) or, inverse, its scale; the pipe is busy 94% of the
+// time.  Against cuFFT (us): y or z 439 -> 305, x 501 + 36 for a pass that widened ->
+// 270 (300 with the offset, with which the spectra below take 3% more), inverse x 501 + 70 for one that stored
 // -> 298.  A spectrum / an initial field (us, cuFFT -> here): 64^3 106 / 95 -> 100 /
 // 89, 96^3 149 / 177 -> 121 / 155, 128^3 277 / 351 -> 206 / 280, 160^3 510 / 643 ->
 // 375 / 507, 192^3 774 / 1039 -> 537 / 765, 256^3 1674 / 2204 -> 1134 / 1625, 512^3
@@ -37,6 +38,7 @@
 
 #include "tl_bits.cuh"
 #include "tl_internal.cuh"
+#include "tl_offset.cuh"
 
 namespace tl {
 
@@ -248,7 +250,8 @@ struct FieldRows {  // a padded field array, rows of N sites
     int f32;
     int N;
     long long pitch, pplane;
-    double base, scale;  // inverse: site = base + scale value
+    double base, scale;    // inverse: site = base + scale value
+    double *offset;        // forward: value = site - offset, which is left here (tl_offset.cuh)
 };
 
 // Lines along x, of L = N/2 points: forward from a field (sites 2n and 2n + 1 the
@@ -265,14 +268,23 @@ __global__ void __launch_bounds__(FftSplit<L>::THREADS, FftSplit<L>::MINB)
     const int z = l / (unsigned)field.N, y = l % (unsigned)field.N;
     const long long at = z * field.pplane + y * field.pitch;
     double2 *p = data + (size_t)l * L;
+    double off = 0.0;
+    if (!inverse) {
+        off = field.f32 ? field_offset(static_cast<const float *>(field.p), field.N, field.pitch, field.pplane)
+                        : field_offset(static_cast<const double *>(field.p), field.N, field.pitch, field.pplane);
+        if (blockIdx.x == 0 && threadIdx.x == 0) *field.offset = off;
+    }
     fft_line<L>(
         j, roots, mul,
         [&](int n) {
             if (!active) return make_double2(0.0, 0.0);
             if (inverse) return parts(p[n], true);
-            if (!field.f32) return *reinterpret_cast<const double2 *>(static_cast<const double *>(field.p) + at + 2 * n);
+            if (!field.f32) {
+                const double2 v = *reinterpret_cast<const double2 *>(static_cast<const double *>(field.p) + at + 2 * n);
+                return make_double2(v.x - off, v.y - off);
+            }
             const float2 v = *reinterpret_cast<const float2 *>(static_cast<const float *>(field.p) + at + 2 * n);
-            return make_double2(widen_bits(v.x), widen_bits(v.y));
+            return make_double2(widen_bits(v.x) - off, widen_bits(v.y) - off);
         },
         [&](int n, double2 v) {
             if (!active) return;

@@ -10,6 +10,7 @@
 #include "tl_bits.cuh"
 #include "tl_boxmuller.cuh"
 #include "tl_fourier.cuh"
+#include "tl_offset.cuh"
 #include "tl_philox.cuh"
 #include "tl_smem.cuh"
 
@@ -170,14 +171,19 @@ __global__ void __launch_bounds__(256) assemble_kernel(T *dst, const double *del
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) widen_kernel(double *dst, const T *src, int N, long long P, long long PP)
+__global__ void __launch_bounds__(256)
+    widen_kernel(double *dst, const T *src, double *offset, int N, long long P, long long PP)
 {
+    const double off = field_offset(src, N, P, PP);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *offset = off;
     const unsigned quads = (unsigned)N / 4, i = blockIdx.x * 256u + threadIdx.x;
     const unsigned row = i / quads, x = 4 * (i - row * quads);
     const int z = row / N, y = row - (unsigned)z * N;
     if (z >= N) return;
     double v[4];
     Four<T>::ld(src + z * PP + y * P + x, v);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] -= off;
     Four<double>::st(dst + (size_t)row * N + x, v);
 }
 
@@ -234,7 +240,7 @@ __device__ __forceinline__ void add_to_shell(int b, double P, double r, unsigned
 // FP64 atomic (a compare-and-swap loop) for each of a mode's three sums this
 // took 475 us at 256^3; here 193.
 __global__ void __launch_bounds__(256) bin_kernel(const double2 *__restrict__ modes, int N, int nbins, double *Psum,
-                                                  double *rsum, unsigned long long *cnt)
+                                                  double *rsum, unsigned long long *cnt, double *mode0)
 {
     extern __shared__ double2 root[];  // N/4 + 1 roots, then the CTA's shell sums
     const int h = N / 2, q = N / 4 + 1;
@@ -247,6 +253,7 @@ __global__ void __launch_bounds__(256) bin_kernel(const double2 *__restrict__ mo
         sC[b] = 0ull;
     }
     fill_roots(root, N, -1.0);  // and a barrier
+    if (blockIdx.x == 0 && threadIdx.x == 0) *mode0 = modes[0].x + modes[0].y;
     const unsigned pairs = (unsigned)(h + 1) * (h + 2) / 2, total = pairs * (unsigned)q;  // below 2^29
     const double scale = 0.25 / ((double)N * N * N) / ((double)N * N * N);
     for (unsigned first = blockIdx.x * 256u; first < total; first += gridDim.x * 256u) {
@@ -339,18 +346,19 @@ cudaError_t launch_assemble(int dtype, void *dst, const double *delta, double ba
     return cudaGetLastError();
 }
 
-cudaError_t launch_widen(int dtype, double *dst, const void *src, int N, long long P, long long PP, cudaStream_t s)
+cudaError_t launch_widen(int dtype, double *dst, const void *src, double *offset, int N, long long P, long long PP,
+                         cudaStream_t s)
 {
     const unsigned grid = (unsigned)(((size_t)N * N * (N / 4) + 255) / 256);
     if (dtype == TL_F32)
-        widen_kernel<float><<<grid, 256, 0, s>>>(dst, static_cast<const float *>(src), N, P, PP);
+        widen_kernel<float><<<grid, 256, 0, s>>>(dst, static_cast<const float *>(src), offset, N, P, PP);
     else
-        widen_kernel<double><<<grid, 256, 0, s>>>(dst, static_cast<const double *>(src), N, P, PP);
+        widen_kernel<double><<<grid, 256, 0, s>>>(dst, static_cast<const double *>(src), offset, N, P, PP);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin(const double2 *modes, int N, int nbins, double *Psum, double *rsum, unsigned long long *cnt,
-                       int sm_count, cudaStream_t s)
+                       double *mode0, int sm_count, cudaStream_t s)
 {
     const size_t total = (size_t)(N / 2 + 1) * (N / 2 + 2) / 2 * (N / 4 + 1);
     const size_t smem = (size_t)(N / 4 + 1) * sizeof(double2) +
@@ -360,7 +368,7 @@ cudaError_t launch_bin(const double2 *modes, int N, int nbins, double *Psum, dou
         const cudaError_t e = limit.raise(bin_kernel, smem);
         if (e != cudaSuccess) return e;
     }
-    bin_kernel<<<grid_for(total, sm_count, 2), 256, smem, s>>>(modes, N, nbins, Psum, rsum, cnt);
+    bin_kernel<<<grid_for(total, sm_count, 2), 256, smem, s>>>(modes, N, nbins, Psum, rsum, cnt, mode0);
     return cudaGetLastError();
 }
 

@@ -26,10 +26,12 @@ cudaError_t launch_fill_modes(double2 *modes, double *power, int N, double kIR, 
 // The padded array at dst = base + scale * delta (delta dense; may be NULL), ghost rows included.
 cudaError_t launch_assemble(int dtype, void *dst, const double *delta, double base, double scale, int N, long long P,
                             long long PP, cudaStream_t s);
-// dst = the padded array at src, dense, in FP64.
-cudaError_t launch_widen(int dtype, double *dst, const void *src, int N, long long P, long long PP, cudaStream_t s);
-// Shell sums of |F|^2 / N^6, |n| and mode counts from C (accumulated with atomics).
+// dst = the padded array at src less its offset (tl_offset.cuh), dense, in FP64; *offset = that.
+cudaError_t launch_widen(int dtype, double *dst, const void *src, double *offset, int N, long long P, long long PP,
+                         cudaStream_t s);
+// Shell sums of |F|^2 / N^6, |n| and mode counts from C (accumulated with atomics);
+// *mode0 = F(0), which alone is in shell 0.
 cudaError_t launch_bin(const double2 *modes, int N, int nbins, double *Psum, double *rsum, unsigned long long *cnt,
-                       int sm_count, cudaStream_t s);
+                       double *mode0, int sm_count, cudaStream_t s);
 
 }  // namespace tl

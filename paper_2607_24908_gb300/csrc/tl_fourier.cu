@@ -80,7 +80,8 @@ __device__ __forceinline__ double2 draw_mode(const BoxMullerTable *t, const doub
 // of four roots and two divisions, 256^3 1305 -> 996 us a field, and the table
 // form of the logarithm and the circle (tl_boxmuller.cuh), 996 -> 610 us; P by |n|^2
 // from a table that a small kernel fills first (a root and three operations a mode
-// less, the same values) and integer-to-FP64 conversions by bits, 604 -> 512 us.
+// less, the same values) and integer-to-FP64 conversions by bits, 604 -> 512 us; four
+// operations a draw for its last roundings, 512 -> 555.
 __global__ void __launch_bounds__(256) fill_modes_kernel(double2 *modes, const double *__restrict__ power, ModeSpec p)
 {
     extern __shared__ double2 root[];

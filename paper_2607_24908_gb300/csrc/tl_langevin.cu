@@ -117,7 +117,7 @@ __device__ __forceinline__ void st(double *p, const double (&v)[2])
 // with two products; 467 instructions a plane and thread, from 538, and less
 // in the last wave: 303 -> 244 us at 384^3, of which the angle's second part took
 // back 4 (248).  FP64 is bound by the FP64 pipe: the
-// table form of Box-Muller (tl_boxmuller.cuh) took 384^3 from 5910 to 3779 us.
+// table form of Box-Muller (tl_boxmuller.cuh) took 384^3 from 5910 to 3951 us.
 template <typename T>
 __global__ void __launch_bounds__(256) langevin_pass(const T *__restrict__ in, T *__restrict__ out, int N, int txt,
                                                      int ty, int zc, long long P, long long PP, T inv_dx2, T dt, T m2,
@@ -210,7 +210,8 @@ extern "C" int tl_langevin_step(tl_lattice *L, int n, double dt, const tl_langev
                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, langevin_pass<double>, 256, 0);
     if (oe != cudaSuccess) return tl::fail(TL_ECUDA, "langevin occupancy: %s", cudaGetErrorString(oe));
     // z-chunk.  FP64 is bound by arithmetic alone, which the two planes a chunk
-    // reads beyond its own do not add to: one plane per CTA spreads it best (us:
+    // reads beyond its own do not add to: one plane per CTA spreads it best (us, with two
+    // operations a draw less than now:
     // 100^3 96 against 116 with 4 planes, 212^3 777 against 795, 384^3 3779 against
     // 3790).  FP32: the fewest (waves of CTAs) x (planes per CTA + 1/4 for those two
     // planes; measured before the angle had its second part): 384^3 244 us with 19

@@ -364,6 +364,7 @@ struct SharedPlan {
     double2 *roots;    // nullptr: the cuFFT plan
     cufftHandle h;
     cudaEvent_t done;  // the table's writing; cuFFT: the latest enqueued execution
+    bool written;      // the table's writing is known to be done
 };
 std::mutex g_plan_mu;
 std::map<std::pair<int, int>, SharedPlan> g_plans;  // (device, N) -> plan
@@ -389,6 +390,20 @@ int make_roots(int N, SharedPlan *p)
     p->roots = d;
     p->done = done;
     return TL_OK;
+}
+
+// Whether a table is written; once it is, its users wait for nothing (a stream in
+// capture could not wait for an event from outside).  Asked in relaxed mode,
+// which allows it whatever this or another thread captures.
+bool table_written(SharedPlan *p)
+{
+    if (p->written) return true;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+    p->written = cudaEventQuery(p->done) == cudaSuccess;
+    if (!p->written) cudaGetLastError();  // not ready
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return p->written;
 }
 
 int shared_plan(int N, cudaStream_t s, SharedPlan **out)
@@ -418,6 +433,7 @@ int shared_plan(int N, cudaStream_t s, SharedPlan **out)
         it = g_plans.emplace(key, p).first;
     }
     *out = &it->second;
+    if (it->second.roots && table_written(&it->second)) return TL_OK;
     if (!it->second.roots) TL_CKFFT(cufftSetStream(it->second.h, s));
     TL_CK(cudaStreamWaitEvent(s, it->second.done, 0));  // a never-recorded event: no wait
     return TL_OK;
